@@ -57,6 +57,7 @@ struct RolloutArgs {
   int mlp_warp;     // 1: each warp runs the policy for its own envs (see mlp_forward_warp)
   TcPlan tc;        // grid policies: the tensor-core forward (tc.on = 0 otherwise)
   StagePlan stage;  // the forward with staged weights (stage.on = 0 otherwise)
+  FwdPlan fwd;      // the router's rollout with one simulator thread per env (fwd.on = 0 otherwise)
   // trace replay (arrival_kind TRACE): gaps, types (or null), costs (or null), length
   const uint32_t* tr_gap;
   const uint8_t* tr_type;
@@ -85,6 +86,9 @@ struct PolicyArgs {
 int act_stride_pad(const DevMlp& m, int B, int threads);
 
 cudaError_t launch_rollout(const RolloutArgs& a, cudaStream_t s);
+// rollout_route.cu: the router's rollout with one simulator thread per env
+size_t plan_route(RolloutArgs& a);
+cudaError_t launch_route(const RolloutArgs& a, size_t sh, cudaStream_t s);
 // step_thread.cu: one thread per env for the policy-free modes
 bool step_thread_supported(const RolloutArgs& a);
 cudaError_t launch_step_thread(const RolloutArgs& a, cudaStream_t s);

@@ -1314,10 +1314,6 @@ size_t plan_tc_forward(RolloutArgs& a, int B) {
   return off;
 }
 
-// Weights of at least this many fp32 bytes are staged in shared memory by default
-// (SIMX_STAGE=0 / 1 turns staging off / on for any size); L1 holds smaller ones.
-constexpr size_t kStageMinBytes = 64 * 1024;
-
 // Register tiles of the staged forward, layer by layer: the first of 4x8, 2x8, 4x4, 2x4,
 // 1x8, 1x4 (envs x outputs) whose tiles keep at least 3/4 of the threads busy, else the
 // one that keeps the most busy; false when a layer's tiles outnumber the threads.
@@ -1434,6 +1430,7 @@ static size_t plan_rollout_t(RolloutArgs& a) {
 }
 
 size_t plan_rollout(RolloutArgs& a) {
+  if (const size_t sh = plan_route(a)) return sh;
   const bool route = a.cfg.mode == SIMX_MODE_ROUTE;
   switch (a.G) {
     case 8: return route ? plan_rollout_t<true, 8>(a) : plan_rollout_t<false, 8>(a);
@@ -1483,7 +1480,11 @@ static cudaError_t observe_t(const RolloutArgs& a, cudaStream_t s) {
     }                                                                                  \
   } while (0)
 
-cudaError_t launch_rollout(const RolloutArgs& a, cudaStream_t s) { SIMX_DISPATCH(rollout_t, a, s); }
+cudaError_t launch_rollout(const RolloutArgs& a0, cudaStream_t s) {
+  RolloutArgs a = a0;
+  if (const size_t sh = plan_route(a)) return launch_route(a, sh, s);
+  SIMX_DISPATCH(rollout_t, a, s);
+}
 cudaError_t launch_reset(const RolloutArgs& a, cudaStream_t s) { SIMX_DISPATCH(reset_t, a, s); }
 cudaError_t launch_observe(const RolloutArgs& a, cudaStream_t s) { SIMX_DISPATCH(observe_t, a, s); }
 

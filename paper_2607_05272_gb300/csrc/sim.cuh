@@ -67,6 +67,30 @@ struct StagePlan {
   int te[SIMX_MAX_LAYERS], to[SIMX_MAX_LAYERS];   // register tile: envs x outputs
 };
 
+// Policies of at least this many fp32 weight bytes have their weights staged in shared
+// memory by default (SIMX_STAGE=0 / 1 turns staging off / on for any size); L1 holds smaller
+// ones.
+constexpr size_t kStageMinBytes = 64 * 1024;
+
+// The block forward of fwd_block.cuh: S stages of cb bytes, chunks of rpc[l] weight rows,
+// register tiles te[l] x to[l]; activation row stride ld.  Byte offsets are inside the
+// kernel's dynamic shared memory.
+struct FwdPlan {
+  int on, big;                 // big: the kernel with 8 x 8 tiles
+  int S, n;
+  uint32_t cb, off, bar_off;   // stages, then 2 S mbarriers (8 B each) and the timeout flag (4 B)
+  uint32_t st_off, red_off;    // env words, softmax partials
+  int ld, ex_row;              // activation row stride, first row of the exponentials
+  int ne_shift;                // log2 of the envs per block
+  uint32_t bias_off;           // the biases of every layer, layer l's from float boff[l]
+  int boff[SIMX_MAX_LAYERS];
+  uint32_t part_off;           // partial results of the servers, S_PARTS words per thread
+  int sms;                     // blocks of one wave index (rotates the warps' roles)
+  int side_layer, side_vt;     // layer beside whose products side work runs (-1: none), from thread
+  int rpc[SIMX_MAX_LAYERS], cnt[SIMX_MAX_LAYERS];
+  int te[SIMX_MAX_LAYERS], to[SIMX_MAX_LAYERS];
+};
+
 template <int G>
 struct Grp {
   uint32_t lane, gl, gi, mask;

@@ -10,98 +10,19 @@
 // those of the lane-group kernel (rollout.cu) and of the oracle, step for step.
 #include <cstdint>
 
+#include "env_thread.cuh"
 #include "kernels.h"
 
 namespace simx {
 
 namespace {
 
+using namespace envt;
+
 template <int K>
-struct TEnv {
-  uint32_t now, tg, cj, cT, swi, swT, mst, ep, epo, pt, pty, pc;
-  uint32_t narr, ndrop, ndisp, nbat, tld, prev, nlast, tlast, na0, na1, nd0, nd1, status, events;
-  uint64_t swait;
-  float lmw, rate, ep_factor;
-  uint32_t ep_cached;
+struct TEnv : TScal {
   uint32_t busy[K], bsize[K], qh0[K], qh1[K], qc0[K], qc1[K];
 };
-
-__device__ __forceinline__ uint32_t t_add(uint32_t a, uint64_t b, uint32_t& status) {
-  const uint64_t s = (uint64_t)a + b;
-  if (s >= kTimeLimit) {
-    status |= kStTime;
-    return kTimeLimit;
-  }
-  return (uint32_t)s;
-}
-
-struct Ctx {
-  const RolloutArgs& A;
-  uint32_t env;
-  uint32_t* ring;  // this env's rings [K][T][cap]
-  uint32_t* cost;  // this env's cost rings [K][cap] or null
-};
-
-__device__ __forceinline__ uint32_t t_type(const simx_config& c, uint32_t w1) {
-  return (c.n_types > 1 && (w1 >> 8) >= c.type0_thr) ? 1u : 0u;
-}
-
-__device__ __forceinline__ uint32_t t_cost(const simx_config& c, uint32_t w3) {
-  const float E = expo1(w3);
-  if (c.cost_kind == 0) return duration_us(__fmul_rn(c.cost_scale_us, det_exp(__fmul_rn(c.pareto_inv_alpha, E))));
-  return duration_us(__fmul_rn(c.cost_scale_us, E));
-}
-
-template <int K>
-__device__ __forceinline__ bool t_count(TEnv<K>& s) {
-  if (++s.events > kEventCap) {
-    s.status |= kStEvent;
-    return true;
-  }
-  return false;
-}
-
-template <int K>
-__device__ void t_switches(const Ctx& x, TEnv<K>& s, uint32_t limit) {
-  if (x.A.cfg.n_mod_states < 2) return;
-  while (s.swT <= limit) {
-    if (t_count(s)) return;
-    s.mst ^= 1u;
-    s.swi += 1u;
-    if (x.A.cfg.dwell_kind == 1) {  // fixed dwell: a square wave
-      s.swT = t_add(s.swT, duration_us(x.A.cfg.dwell_mean_us), s.status);
-    } else {
-      const U4 w = philox(s.swi, x.env, kStreamSwitch, 0u, x.A.key0, x.A.key1);
-      s.swT = t_add(s.swT, duration_us(__fmul_rn(x.A.cfg.dwell_mean_us, expo1(w.x))), s.status);
-    }
-  }
-}
-
-// Candidate s.cj: its Philox words and its time (a drawn gap, or under trace replay,
-// TR, entry cj mod n of the trace).  TR is a template parameter so that the generated-
-// arrival kernels carry none of the trace code.
-template <int K, bool TR>
-__device__ __forceinline__ uint32_t t_cand(const Ctx& x, TEnv<K>& s, U4& w) {
-  w = philox(s.cj, x.env, kStreamArrival, 0u, x.A.key0, x.A.key1);
-  const uint32_t gap = TR ? x.A.tr_gap[s.cj % x.A.tr_n]
-                          : duration_us(__fmul_rn(x.A.cfg.cand_mean_gap_us, expo1(w.x)));
-  return t_add(s.cT, gap, s.status);
-}
-
-// Type and cost of candidate j: the trace's when it has them, else drawn.
-template <bool TR>
-__device__ __forceinline__ uint32_t t_cand_type(const RolloutArgs& A, uint32_t j, uint32_t w1) {
-  if (TR && A.tr_type) {
-    const uint32_t t = A.tr_type[j % A.tr_n];
-    return t < A.cfg.n_types ? t : A.cfg.n_types - 1u;
-  }
-  return t_type(A.cfg, w1);
-}
-
-template <bool TR>
-__device__ __forceinline__ uint32_t t_cand_cost(const RolloutArgs& A, uint32_t j, uint32_t w3) {
-  return (TR && A.tr_cost) ? A.tr_cost[j % A.tr_n] : t_cost(A.cfg, w3);
-}
 
 // SINGLE mode: an accepted candidate joins its type's FIFO or is dropped.
 template <int K, bool TR>
@@ -129,7 +50,7 @@ template <int K, bool TR>
 __device__ void t_advance(const Ctx& x, TEnv<K>& s, uint32_t target) {
   for (;;) {
     U4 w;
-    const uint32_t T = t_cand<K, TR>(x, s, w);
+    const uint32_t T = t_cand<TR>(x, s, w);
     if (T > target) break;
     if (t_count(s)) return;
     t_switches(x, s, T);
@@ -144,7 +65,7 @@ template <int K, bool TR>
 __device__ void t_jump(const Ctx& x, TEnv<K>& s) {
   for (;;) {
     U4 w;
-    const uint32_t T = t_cand<K, TR>(x, s, w);
+    const uint32_t T = t_cand<TR>(x, s, w);
     if (t_count(s)) return;
     t_switches(x, s, T);
     const bool acc = t_consume<K, TR>(x, s, w, T);
@@ -158,80 +79,20 @@ __device__ void t_jump(const Ctx& x, TEnv<K>& s) {
   }
 }
 
-// ROUTE mode: the next arrival into the pending slot.
-template <int K, bool TR>
-__device__ void t_next_arrival(const Ctx& x, TEnv<K>& s) {
-  const simx_config& c = x.A.cfg;
-  for (;;) {
-    if (t_count(s)) return;
-    U4 w;
-    if (TR || c.arrival_kind != SIMX_ARR_DIURNAL) {  // THINNED or TRACE
-      const uint32_t T = t_cand<K, TR>(x, s, w);
-      t_switches(x, s, T);
-      const bool acc = (w.z >> 8) < c.accept_thr[s.mst];
-      const uint32_t j = s.cj;
-      s.cj += 1u;
-      s.cT = T;
-      if (!acc) continue;
-      s.pty = t_cand_type<TR>(x.A, j, w.y);
-      s.pc = ((int32_t)s.pty == c.cost_type) ? t_cand_cost<TR>(x.A, j, w.w) : 0u;
-      s.pt = T;
-      s.narr += 1u;
-      return;
-    }
-    if (s.ep_cached != s.ep) {
-      const U4 we = philox(s.ep, x.env, kStreamEpoch, 0u, x.A.key0, x.A.key1);
-      s.ep_factor = det_exp(__fmul_rn(c.burst_sigma, normal01(we.x, we.y)));
-      s.ep_cached = s.ep;
-    }
-    const float rate = __fmul_rn(c.diurnal_rate[(s.ep + s.epo) % c.diurnal_len], s.ep_factor);
-    const float mean = __fdiv_rn(1.0e6f, rate);
-    w = philox(s.cj, x.env, kStreamArrival, 0u, x.A.key0, x.A.key1);
-    const uint32_t gap = duration_us(__fmul_rn(mean, expo1(w.x)));
-    s.cj += 1u;
-    const uint64_t end = (uint64_t)(s.ep + 1u) * (uint64_t)c.epoch_us;
-    if ((uint64_t)s.cT + gap < end) {
-      s.cT = t_add(s.cT, gap, s.status);
-      s.pt = s.cT;
-      s.pty = t_type(c, w.y);
-      s.pc = ((int32_t)s.pty == c.cost_type) ? t_cost(c, w.w) : 0u;
-      s.narr += 1u;
-      return;
-    }
-    if (end >= kTimeLimit) {
-      s.status |= kStTime;
-      s.cT = kTimeLimit;
-    } else {
-      s.cT = (uint32_t)end;
-    }
-    s.ep += 1u;
-  }
-}
-
-// Batch time L on server k scaled by its speed s/16, rounded to the nearest microsecond.
-__device__ __forceinline__ uint64_t t_speed(const simx_config& c, int k, uint64_t L) {
-  const uint64_t s = c.srv_speed16[k] ? c.srv_speed16[k] : 16u;
-  return (L * s + 8u) >> 4;
-}
-
 // ROUTE mode: one server's queue state, selected out of the register arrays by unrolled
 // selects so that the batch start below is emitted once per call site instead of once per
 // server (the K-fold copies made the kernel's instruction fetch its largest stall).
-struct Srv {
-  uint32_t busy, bsize, qh0, qc0, qh1, qc1;
-};
-
 template <int K>
-__device__ __forceinline__ Srv srv_get(const TEnv<K>& s, int i) {
-  Srv r{s.busy[0], s.bsize[0], s.qh0[0], s.qc0[0], s.qh1[0], s.qc1[0]};
+__device__ __forceinline__ TSrv srv_get(const TEnv<K>& s, int i) {
+  TSrv r{s.busy[0], s.bsize[0], s.qh0[0], s.qc0[0], s.qh1[0], s.qc1[0]};
 #pragma unroll
   for (int k = 1; k < K; ++k)
-    if (i == k) r = Srv{s.busy[k], s.bsize[k], s.qh0[k], s.qc0[k], s.qh1[k], s.qc1[k]};
+    if (i == k) r = TSrv{s.busy[k], s.bsize[k], s.qh0[k], s.qc0[k], s.qh1[k], s.qc1[k]};
   return r;
 }
 
 template <int K>
-__device__ __forceinline__ void srv_put(TEnv<K>& s, int i, const Srv& r) {
+__device__ __forceinline__ void srv_put(TEnv<K>& s, int i, const TSrv& r) {
 #pragma unroll
   for (int k = 0; k < K; ++k)
     if (i == k) {
@@ -244,51 +105,6 @@ __device__ __forceinline__ void srv_put(TEnv<K>& s, int i, const Srv& r) {
     }
 }
 
-// ROUTE mode: server i (state r) starts a batch at time st (the oldest-head type, tie:
-// type 0).
-template <int K>
-__device__ __forceinline__ void t_start(const Ctx& x, TEnv<K>& s, Srv& r, int i, uint32_t st,
-                                        uint32_t& stn, uint64_t& w0, uint64_t& w1) {
-  const simx_config& c = x.A.cfg;
-  const uint32_t cap = c.queue_cap, T = c.n_types;
-  uint32_t* rs = x.ring + (size_t)i * T * cap;
-  uint32_t h;
-  if (r.qc0 > 0u && r.qc1 > 0u) {
-    h = rs[cap + r.qh1] < rs[r.qh0] ? 1u : 0u;
-  } else if (r.qc0 > 0u) {
-    h = 0u;
-  } else if (r.qc1 > 0u) {
-    h = 1u;
-  } else {
-    return;
-  }
-  const uint32_t qn = h ? r.qc1 : r.qc0;
-  const uint32_t head = h ? r.qh1 : r.qh0;
-  const uint32_t n = r.bsize < qn ? r.bsize : qn;
-  const bool costed = (int32_t)h == c.cost_type;
-  uint64_t W = 0, csum = 0;
-  for (uint32_t j = 0; j < n; ++j) {
-    const uint32_t slot = (head + j) & (cap - 1u);
-    W += (uint64_t)(st - rs[h * cap + slot]);
-    if (costed) csum += x.cost[(size_t)i * cap + slot];
-  }
-  if (h) {
-    r.qh1 = (head + n) & (cap - 1u);
-    r.qc1 -= n;
-  } else {
-    r.qh0 = (head + n) & (cap - 1u);
-    r.qc0 -= n;
-  }
-  const uint64_t L = costed ? (uint64_t)c.alpha_us[h] + csum
-                            : (uint64_t)c.alpha_us[h] + (uint64_t)c.beta_us[h] * n;
-  r.busy = t_add(st, t_speed(c, i, L), s.status);
-  stn += n;
-  if (h) w1 += W; else w0 += W;
-  s.ndisp += n;
-  s.swait += W;
-  s.nbat += 1u;
-}
-
 template <int K>
 __device__ __forceinline__ uint32_t t_queued(const TEnv<K>& s) {
   uint32_t q = 0;
@@ -298,12 +114,6 @@ __device__ __forceinline__ uint32_t t_queued(const TEnv<K>& s) {
 }
 
 // Observation (Sec. 4.1; the layouts of rollout.cu) into obs[d * ld].
-// q / cap for a power-of-two capacity: multiplying by the exact reciprocal 2^-k gives
-// the bits of the IEEE division (no rounding either way for these small integers).
-__device__ __forceinline__ float over_cap(uint32_t q, float inv_cap) {
-  return __fmul_rn(__uint2float_rn(q), inv_cap);
-}
-
 template <bool ROUTE, int K>
 __device__ void t_observe(const Ctx& x, const TEnv<K>& s, float* o, int64_t ld) {
   const simx_config& c = x.A.cfg;
@@ -543,12 +353,12 @@ __global__ void __launch_bounds__(128, MINB) k_step_thread(const __grid_constant
           go = s.busy[k] <= now;
         }
         if (go) {  // the routed-to server is free: it starts a batch now
-          Srv r = srv_get<K>(s, (int)kk);
-          t_start<K>(x, s, r, (int)kk, now, stn, w0, w1);
+          TSrv r = srv_get<K>(s, (int)kk);
+          t_start<1u>(x, s, r, (int)kk, now, stn, w0, w1);
           srv_put<K>(s, (int)kk, r);
         }
         qafter = t_queued(s);
-        t_next_arrival<K, TR>(x, s);
+        t_next_arrival<TR>(x, s);
         uint32_t gap = s.pt - now;
         if (gap < 1u) gap = 1u;
         const float inst = __fdiv_rn(1.0e6f, __uint2float_rn(gap));
@@ -561,8 +371,8 @@ __global__ void __launch_bounds__(128, MINB) k_step_thread(const __grid_constant
           for (int j = K - 1; j >= 0; --j)
             if (s.busy[j] <= s.pt && (s.qc0[j] + s.qc1[j]) > 0u) k = j;
           if (k < 0) break;
-          Srv r = srv_get<K>(s, k);
-          t_start<K>(x, s, r, k, r.busy, stn, w0, w1);
+          TSrv r = srv_get<K>(s, k);
+          t_start<1u>(x, s, r, k, r.busy, stn, w0, w1);
           srv_put<K>(s, k, r);
         }
         s.now = s.pt;
