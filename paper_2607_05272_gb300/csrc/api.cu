@@ -186,17 +186,27 @@ simx_status pack_mlp(const simx_mlp* m, Packed& P, DevMlp& out, cudaStream_t s) 
   }
   std::memset(&out, 0, sizeof(out));
   float* p = P.buf;
+  RepackArgs r;
+  std::memset(&r, 0, sizeof(r));
+  r.n_layers = m->n_layers;
   for (int l = 0; l < m->n_layers; ++l) {
     const int K = m->dims[l], N = m->dims[l + 1];
     float* Wt = p;
     float* bias = p + (size_t)K * npad[l + 1];
-    cudaError_t e = launch_repack(m->W[l], m->b[l], N, K, npad[l + 1], Wt, bias, s);
-    if (e != cudaSuccess) return cuda_fail(e, "repack");
+    r.W[l] = m->W[l];
+    r.b[l] = m->b[l];
+    r.Wt[l] = Wt;
+    r.bias[l] = bias;
+    r.N[l] = N;
+    r.K[l] = K;
+    r.npad[l] = npad[l + 1];
     out.Wt[l] = Wt;
     out.bias[l] = bias;
     out.act[l] = (l + 1 < m->n_layers) ? m->act[l] : -1;  // -1: no activation (output layer)
     p = bias + npad[l + 1];
   }
+  const cudaError_t e = launch_repack(r, s);
+  if (e != cudaSuccess) return cuda_fail(e, "repack");
   for (int l = 0; l <= m->n_layers; ++l) {
     out.dims[l] = m->dims[l];
     out.npad[l] = l ? npad[l] : m->dims[0];

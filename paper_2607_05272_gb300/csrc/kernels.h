@@ -77,6 +77,7 @@ struct PolicyArgs {
   float* logp;
   int maxd4, apad;
   int G, threads;
+  FwdPlan fwd;      // the block forward (fwd_block.cuh)
 };
 
 // Padding of the block's activation rows: 4 (16-byte rows) when some layer takes the
@@ -97,8 +98,30 @@ cudaError_t launch_observe(const RolloutArgs& a, cudaStream_t s);
 cudaError_t launch_save(const DevState& st, int32_t cost_type, uint64_t words, uint32_t* out, cudaStream_t s);
 cudaError_t launch_load(const DevState& st, int32_t cost_type, uint64_t words, const uint32_t* in, cudaStream_t s);
 cudaError_t launch_stats(const DevState& st, unsigned long long* out, cudaStream_t s);
-cudaError_t launch_repack(const float* W, const float* b, int N, int K, int Npad, float* Wt, float* bias, cudaStream_t s);
+// W_l [N][K] -> Wt_l [K][Npad], b_l -> bias_l [Npad] for every layer of a policy, in one launch
+struct RepackArgs {
+  const float* W[SIMX_MAX_LAYERS];
+  const float* b[SIMX_MAX_LAYERS];
+  float* Wt[SIMX_MAX_LAYERS];
+  float* bias[SIMX_MAX_LAYERS];
+  int N[SIMX_MAX_LAYERS], K[SIMX_MAX_LAYERS], npad[SIMX_MAX_LAYERS];
+  int n_layers;
+};
+cudaError_t launch_repack(const RepackArgs& r, cudaStream_t s);
 cudaError_t launch_policy_forward(const PolicyArgs& p, cudaStream_t s);
+// policy_forward.cu: the batched forward of FP32 policies, and the plans that it shares with the
+// router's rollout.
+// Register tiles of layer l: the largest of 8x8 (big), 4x8, 2x8, 4x4, 2x4, 1x4 that gives `pct`
+// percent of the threads a tile, else the one with the most tiles; also sets P.ne_shift.
+bool fwd_pick_tiles(const DevMlp& m, int NE, int threads, bool big, int pct, FwdPlan& P);
+// Places of the biases after P.bias_off; returns their bytes.
+size_t fwd_plan_biases(const DevMlp& m, FwdPlan& P);
+// Two weight stages from byte `off` on within `budget` bytes of shared memory (at least one row
+// each), and the chunks.
+bool fwd_plan_stages(const DevMlp& m, size_t off, size_t budget, FwdPlan& P);
+size_t fwd_smem(const FwdPlan& P);
+bool plan_policy_block(PolicyArgs& p);
+cudaError_t launch_policy_block(const PolicyArgs& p, cudaStream_t s);
 // Sets a.tc (and the activation rows a.maxd4 it needs) when the grid forward of this
 // launch can run on the tensor cores; returns the dynamic shared memory of the launch.
 size_t plan_tc_forward(RolloutArgs& a, int B);

@@ -1210,19 +1210,27 @@ __global__ void k_stats(DevState st, unsigned long long* out) {
   if ((threadIdx.x & 31u) == 0 && sor) atomicOr(reinterpret_cast<unsigned int*>(out + 8), sor);
 }
 
-// W [N][K] row-major -> Wt [K][Npad] (zero-padded columns), b [N] -> bias [Npad].
-__global__ void k_repack(const float* __restrict__ W, const float* __restrict__ b, int N, int K,
-                         int Npad, float* __restrict__ Wt, float* __restrict__ bias) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < K * Npad) {
-    const int k = i / Npad, j = i % Npad;
-    Wt[i] = j < N ? W[(size_t)j * K + k] : 0.0f;
-  }
-  if (i < Npad) bias[i] = i < N ? b[i] : 0.0f;
+// W_l [N][K] row-major -> Wt_l [K][Npad] (zero-padded columns), b_l [N] -> bias_l [Npad], every
+// layer in one launch (blockIdx.z).  32 x 32 tiles go through shared memory, so that both the
+// reads (along k) and the writes (along j) are whole rows.
+__global__ void __launch_bounds__(256) k_repack(const __grid_constant__ RepackArgs R) {
+  __shared__ float tile[32][33];
+  const int l = blockIdx.z, N = R.N[l], K = R.K[l], Np = R.npad[l];
+  const int j0 = 32 * (int)blockIdx.x, k0 = 32 * (int)blockIdx.y;
+  if (j0 >= Np || k0 >= K) return;
+  const float* __restrict__ W = R.W[l];
+  const int tx = (int)threadIdx.x & 31, ty = (int)threadIdx.x >> 5;
+  for (int i = ty; i < 32; i += 8)
+    tile[i][tx] = (j0 + i < N && k0 + tx < K) ? W[(size_t)(j0 + i) * K + k0 + tx] : 0.0f;
+  __syncthreads();
+  for (int i = ty; i < 32; i += 8)
+    if (k0 + i < K && j0 + tx < Np) R.Wt[l][(size_t)(k0 + i) * Np + j0 + tx] = tile[tx][i];
+  if (k0 == 0 && ty == 0 && j0 + tx < Np) R.bias[l][j0 + tx] = j0 + tx < N ? R.b[l][j0 + tx] : 0.0f;
 }
 
-// Batched policy forward (Sec. 4.2) over observation columns [D][ld]: a block of
-// B = blockDim.x / G columns runs the block-wide MLP, then each column's G lanes
+// Batched forward (Sec. 4.2) of grid policies, and of FP32 ones whose output layer has too many
+// rows for the register tiles of policy_forward.cu (above 128, off a multiple of 8), over
+// observation columns [D][ld]: a block of B = blockDim.x / G columns runs the block-wide MLP, then each column's G lanes
 // sample.  Every lane stays alive for the block barriers.
 template <int G>
 __global__ void __launch_bounds__(kMaxThreads)
@@ -1508,10 +1516,13 @@ cudaError_t launch_stats(const DevState& st, unsigned long long* out, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t launch_repack(const float* W, const float* b, int N, int K, int Npad, float* Wt,
-                          float* bias, cudaStream_t s) {
-  const int n = K * Npad > Npad ? K * Npad : Npad;
-  k_repack<<<(n + 255) / 256, 256, 0, s>>>(W, b, N, K, Npad, Wt, bias);
+cudaError_t launch_repack(const RepackArgs& r, cudaStream_t s) {
+  int n = 0, k = 0;
+  for (int l = 0; l < r.n_layers; ++l) {
+    n = r.npad[l] > n ? r.npad[l] : n;
+    k = r.K[l] > k ? r.K[l] : k;
+  }
+  k_repack<<<dim3((unsigned)((n + 31) / 32), (unsigned)((k + 31) / 32), (unsigned)r.n_layers), 256, 0, s>>>(r);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1526,7 +1537,9 @@ static cudaError_t policy_forward_t(const PolicyArgs& p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_policy_forward(const PolicyArgs& p, cudaStream_t s) {
+cudaError_t launch_policy_forward(const PolicyArgs& p0, cudaStream_t s) {
+  PolicyArgs p = p0;
+  if (plan_policy_block(p)) return launch_policy_block(p, s);
   switch (p.G) {
     case 8: return policy_forward_t<8>(p, s);
     case 16: return policy_forward_t<16>(p, s);

@@ -289,14 +289,7 @@ __device__ __forceinline__ void phase_step(const RolloutArgs& A, float* smem, in
   // the softmax, G threads per env: the largest logit, then the exponentials
   const float* z = w.X + w.slot;
   float* ex = w.ex + w.slot;
-  float mx = -__uint_as_float(0x7F800000u);
-  for (int i = w.part; i < NA; i += G) mx = fmaxf(mx, z[i * ld]);
-  w.red[w.vt] = mx;
-  __syncthreads();
-  mx = w.red[w.slot];
-  for (int q = 1; q < G; ++q) mx = fmaxf(mx, w.red[q * w.NE + w.slot]);
-  for (int i = w.part; i < NA; i += G) ex[i * ld] = fwd::exp_flat(__fsub_rn(z[i * ld], mx));
-  __syncthreads();
+  const float mx = fwd::softmax_parts(z, ex, w.red, NA, ld, w.vt, w.part, w.slot, G, w.NE);
   const SmEnv& S = w.S;
   const bool owner = w.part == 0 && w.live;   // the env's thread
   const size_t env = w.live ? w.env : 0u;
@@ -305,29 +298,8 @@ __device__ __forceinline__ void phase_step(const RolloutArgs& A, float* smem, in
   const int64_t o = (int64_t)t * A.ld + w.env;
   if (owner) {
     if (P.side_layer < 0) look_ahead<TR>(x, S);
-    // the partial sums in index order replace the exponentials; the draw is the first above
-    // u times the last (they never decrease), else the last action
-    float sum = 0.0f;
-    for (int i0 = 0; i0 < NA; i0 += 8) {   // 8 loads before the stores that might alias them
-      float e8[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) e8[i] = i0 + i < NA ? ex[(i0 + i) * ld] : 0.0f;
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (i0 + i < NA) {
-          sum = __fadd_rn(sum, e8[i]);
-          ex[(i0 + i) * ld] = sum;
-        }
-    }
-    int a = 0;
-    if (A.policy_mode == SIMX_POLICY_ARGMAX) {
-      for (int i = NA - 1; i >= 0; --i)
-        if (z[i * ld] == mx) a = i;
-    } else {
-      const float thr = __fmul_rn(u_open1(S[W_U]), sum);
-#pragma unroll 8
-      for (int i = 0; i + 1 < NA; ++i) a += ex[i * ld] > thr ? 0 : 1;
-    }
+    float sum;
+    const int a = fwd::draw(z, ex, NA, ld, mx, A.policy_mode == SIMX_POLICY_ARGMAX, S[W_U], sum);
     const fwd::Pipe p = fwd::pipe_at(reinterpret_cast<unsigned char*>(smem), P);
     route_apply(x, S, a, *p.flag ? SIMX_DEV_COPY_TIMEOUT : 0u);
     if (A.action) A.action[o] = (uint8_t)a;
@@ -444,38 +416,6 @@ __global__ void __launch_bounds__(NT, MINB) k_route(const __grid_constant__ Roll
 
 namespace {
 
-// Register tiles of layer l: the largest of 8x8 (big), 4x8, 2x8, 4x4, 2x4, 1x4 that gives
-// `pct` percent of the threads a tile, else the one with the most tiles.
-bool pick_tiles(const DevMlp& m, int NE, int threads, bool big, FwdPlan& P) {
-  static const int shapes[6][2] = {{8, 8}, {4, 8}, {2, 8}, {4, 4}, {2, 4}, {1, 4}};
-  // 8x8 tiles on half of the threads beat 4x8 on all of them for 256-wide layers (c4, 65,536
-  // envs: 320 against 340 us per step); narrower layers want every thread (c3, 16,384 envs:
-  // 41 us per step with 2x8 tiles on all threads, 50 with 4x8 on half)
-  const int pct = big ? 40 : 75;
-  for (int l = 0; l < m.n_layers; ++l) {
-    const int N = m.dims[l + 1], Np = m.npad[l + 1];
-    int best = -1, best_nt = 0;
-    for (int q = big ? 0 : 1; q < 6; ++q) {
-      const int te = shapes[q][0], to = shapes[q][1];
-      if (NE % te != 0 || Np % to != 0) continue;
-      const int nt = (NE / te) * ((N + to - 1) / to);
-      if (nt > threads) continue;
-      if (100 * nt >= pct * threads) {
-        best = q;
-        break;
-      }
-      if (nt > best_nt) {
-        best_nt = nt;
-        best = q;
-      }
-    }
-    if (best < 0) return false;
-    P.te[l] = shapes[best][0];
-    P.to[l] = shapes[best][1];
-  }
-  return true;
-}
-
 const void* pick_kernel(const RolloutArgs& a) {
   const bool tr = a.cfg.arrival_kind == SIMX_ARR_TRACE;
   if (a.fwd.big) return tr ? (const void*)k_route<true, 256, 2, true> : (const void*)k_route<false, 256, 2, true>;
@@ -502,9 +442,8 @@ size_t plan_route(RolloutArgs& a) {
   size_t wbytes = 0;
   for (int l = 0; l < m.n_layers; ++l) wbytes += (size_t)m.dims[l] * m.npad[l + 1] * sizeof(float);
   if (force < 0 && wbytes < kStageMinBytes) return 0;
-  int maxd = 0, maxnp = 0, nb = 0;
+  int maxd = 0;
   for (int l = 0; l <= m.n_layers; ++l) maxd = m.dims[l] > maxd ? m.dims[l] : maxd;
-  for (int l = 1; l <= m.n_layers; ++l) maxnp = m.npad[l] > maxnp ? m.npad[l] : maxnp;
   const bool wide = maxd > 128;
   // Envs per block.  Every block streams the whole policy through its stages each step, so few
   // envs per block cost more copying than they win in parallel blocks: 256 threads take 8 envs
@@ -530,9 +469,10 @@ size_t plan_route(RolloutArgs& a) {
   std::memset(&P, 0, sizeof(P));
   const int last = r4(m.dims[m.n_layers]);
   P.big = threads == 256 && wide && NE >= 16;
-  if (!pick_tiles(m, NE, threads, P.big, P)) return 0;
-  while ((1 << P.ne_shift) < NE) ++P.ne_shift;
-  if ((1 << P.ne_shift) != NE) return 0;
+  // 8x8 tiles on half of the threads beat 4x8 on all of them for 256-wide layers (c4, 65,536
+  // envs: 320 against 340 us per step); narrower layers want every thread (c3, 16,384 envs:
+  // 41 us per step with 2x8 tiles on all threads, 50 with 4x8 on half)
+  if (!fwd_pick_tiles(m, NE, threads, P.big, P.big ? 40 : 75, P)) return 0;
   P.ld = NE + 4;
   P.ex_row = last;   // the exponentials follow the logits and the value row
   const int rows = r4(maxd) > last + r4(m.n_actions) ? r4(maxd) : last + r4(m.n_actions);
@@ -550,13 +490,7 @@ size_t plan_route(RolloutArgs& a) {
     off += (size_t)threads * sizeof(float);
   }
   P.bias_off = (uint32_t)off;
-  for (int l = 0; l < m.n_layers; ++l) {
-    P.boff[l] = nb;
-    nb += m.dims[l + 1];
-  }
-  off += (size_t)nb * sizeof(float);
-  off = (off + 127) / 128 * 128;
-  P.off = (uint32_t)off;
+  off += fwd_plan_biases(m, P);
   // Two stages, as large as keeps the blocks per SM that the registers allow: each chunk costs
   // about 500 cycles of waiting and pipeline fill, so fewer and larger ones win over more
   // stages (c4 at 65,536 envs: 2 x 32 KB 320 us per step, 4 x 16 KB 338, 8 x 8 KB 376; c3 at
@@ -566,22 +500,7 @@ size_t plan_route(RolloutArgs& a) {
   int64_t per_sm = (blocks + sm_count() - 1) / sm_count();
   if (per_sm > minb) per_sm = minb;
   const size_t budget = (size_t)(227 * 1024) / (size_t)per_sm - 1024;
-  P.S = 2;
-  uint32_t cb = 32768;
-  while (cb > 2048 && off + (size_t)P.S * cb + 128 > budget) cb -= 1024;
-  if (cb < (uint32_t)maxnp * 4u) cb = (uint32_t)(maxnp * 4 + 127) / 128u * 128u;   // at least one row
-  if (off + (size_t)P.S * cb + 128 > 227 * 1024) return 0;
-  P.cb = cb;
-  for (int l = 0; l < m.n_layers; ++l) {
-    const int K = m.dims[l];
-    int rpc = (int)(cb / (uint32_t)(m.npad[l + 1] * 4));
-    if (rpc >= 16) rpc &= ~7;   // whole passes of the unrolled loop
-    rpc = rpc < K ? rpc : K;
-    P.rpc[l] = rpc;
-    P.cnt[l] = (K + rpc - 1) / rpc;
-    P.n += P.cnt[l];
-  }
-  P.bar_off = (uint32_t)(off + (size_t)P.S * cb);
+  if (!fwd_plan_stages(m, off, budget, P)) return 0;
   P.sms = sm_count();
   // side work beside the deepest layer that leaves NE threads without tiles (the last warp apart)
   P.side_layer = -1;
@@ -598,7 +517,7 @@ size_t plan_route(RolloutArgs& a) {
   a.fwd = P;
   a.G = G;
   a.threads = threads;
-  return P.bar_off + fwd::pipe_bytes(P.S);
+  return fwd_smem(P);
 }
 
 cudaError_t launch_route(const RolloutArgs& a, size_t sh, cudaStream_t s) {
