@@ -9,11 +9,15 @@
 // Large env counts with 16-byte aligned rows take k_returns_wide: one thread owns four
 // adjacent envs for the whole horizon (one pass: every input read once, every output
 // written once, 17 bytes per sample for GAE), loading 8 time steps ahead with 16-byte
-// loads, so a block reads 1 KB of each row per step.  Otherwise:
-// a block owns 32 envs (threadIdx.x) and splits time into S chunks (threadIdx.y).
-// Each thread composes its chunk's map x_{t0} = a x_{t1} + b, one thread per env
-// chains the S maps in shared memory, then every thread replays its chunk from the
-// right carry.  Loads are coalesced across envs; no global scratch is needed.
+// loads, so a block reads 1 KB of each row per step.  Otherwise a block owns 32 envs
+// (threadIdx.x) and S chunks of 8 steps at a time (threadIdx.y), held in registers.  Each thread
+// composes its chunk's map x_{t0} = a x_{t1} + b, one thread per env chains the S maps in shared
+// memory, then every thread replays its chunk from the right carry.  Loads are coalesced across
+// envs; no global scratch is needed.  Bound by HBM: 20.5 us at 16,384 envs x 256, inputs not in
+// L2 (k_returns_long 22.5); 234 us at 60,000 x 1024 (300).  Long horizons of few envs would walk
+// many windows, each a round trip to memory and three barriers: they take k_returns_long, whose
+// threads each read a chunk of up to T / 32 steps twice without a barrier between (4003 envs x
+// 1960: 35 us against 44; 64 x 2048: 20 against 29).
 #include <cstdint>
 
 #include "kernels.h"
@@ -21,9 +25,113 @@
 namespace simx {
 
 constexpr int kRetMaxChunks = 32;
+constexpr int kRetL = 8;   // steps per chunk, held in registers
 
+// One thread's chunk of one window: kRetL steps of one env from step t0 on.  Steps past the
+// horizon stand for the state after it: value `last`, no reward.
+template <bool GAE>
+struct RetChunk {
+  float r[kRetL], v[GAE ? kRetL : 1];
+  uint32_t d;   // bit i: step i ends its segment
+  __device__ __forceinline__ void load(const float* __restrict__ rew, const float* __restrict__ val,
+                                       const uint8_t* __restrict__ done, int64_t t0, int64_t T, int64_t ld,
+                                       int64_t e, bool live, float last) {
+    uint8_t dd[kRetL];
+#pragma unroll
+    for (int i = 0; i < kRetL; ++i) {
+      const bool in = live && t0 + i < T;
+      const int64_t o = (t0 + i) * ld + e;
+      r[i] = in ? rew[o] : 0.0f;
+      dd[i] = in ? done[o] : (uint8_t)0;
+      if (GAE) v[i] = in ? val[o] : last;
+    }
+    d = 0u;
+#pragma unroll
+    for (int i = 0; i < kRetL; ++i) d |= dd[i] ? 1u << i : 0u;
+  }
+};
+
+// A block owns 32 envs and walks the horizon backwards in windows of S chunks of kRetL steps,
+// the next window's loads in flight while this one is chained.  Every input is read once.
+template <bool GAE>
 __global__ void __launch_bounds__(1024)
 k_returns_gae(const float* __restrict__ rew, const float* __restrict__ val,
+              const uint8_t* __restrict__ done, const float* __restrict__ last_val, int64_t T,
+              int64_t E, int64_t ld, float gamma, float lam, float* __restrict__ ret,
+              float* __restrict__ adv) {
+  __shared__ float sa[kRetMaxChunks][32], sb[kRetMaxChunks][32], scarry[kRetMaxChunks][32];
+  __shared__ float sv[kRetMaxChunks + 1][32];   // row j: chunk j's first value; row S: the window after
+  const int x = threadIdx.x, j = threadIdx.y, S = blockDim.y;
+  const int64_t e = (int64_t)blockIdx.x * 32 + x;
+  const bool live = e < E;
+  const float cmul = GAE ? gamma * lam : gamma;
+  const float last = live && last_val ? last_val[e] : 0.0f;
+  const int64_t W = (int64_t)S * kRetL;
+  int64_t t0 = (T + W - 1) / W * W - W + (int64_t)j * kRetL;
+  float carry = GAE ? 0.0f : last;   // (threads of chunk 0) the recurrence entering from the right
+  if (GAE && j == 0) sv[S][x] = last;
+  RetChunk<GAE> c;
+  c.load(rew, val, done, t0, T, ld, e, live, last);
+  for (;;) {
+    RetChunk<GAE> nx;
+    if (t0 >= W) nx.load(rew, val, done, t0 - W, T, ld, e, live, last);
+    if (GAE) {
+      sv[j][x] = c.v[0];
+      __syncthreads();
+    }
+    // this chunk's map x_{t0} = a x_{t1} + b; r becomes delta
+    float vnext = GAE ? sv[j + 1][x] : 0.0f;
+    float a = 1.0f, b = 0.0f;
+#pragma unroll
+    for (int i = kRetL - 1; i >= 0; --i) {
+      const float mask = (c.d >> i) & 1u ? 0.0f : 1.0f;
+      if (GAE) {
+        c.r[i] = c.r[i] + gamma * mask * vnext - c.v[i];
+        vnext = c.v[i];
+      }
+      if (t0 + i < T) {
+        const float cc = cmul * mask;
+        b = c.r[i] + cc * b;
+        a = cc * a;
+      }
+    }
+    sa[j][x] = a;
+    sb[j][x] = b;
+    __syncthreads();
+    if (j == 0) {
+      if (GAE) sv[S][x] = c.v[0];
+#pragma unroll 4
+      for (int q = S - 1; q >= 0; --q) {
+        scarry[q][x] = carry;
+        carry = sb[q][x] + sa[q][x] * carry;
+      }
+    }
+    __syncthreads();
+    // replay with the carry that enters the chunk from the right
+    float y = scarry[j][x];
+#pragma unroll
+    for (int i = kRetL - 1; i >= 0; --i) {
+      if (live && t0 + i < T) {
+        const float mask = (c.d >> i) & 1u ? 0.0f : 1.0f;
+        const int64_t o = (t0 + i) * ld + e;
+        y = c.r[i] + cmul * mask * y;
+        if (GAE) {
+          adv[o] = y;
+          ret[o] = y + c.v[i];
+        } else {
+          ret[o] = y;
+          if (adv) adv[o] = y;
+        }
+      }
+    }
+    if (t0 < W) break;   // the same for every thread of the block: W divides each window's start
+    t0 -= W;
+    c = nx;
+  }
+}
+
+__global__ void __launch_bounds__(1024)
+k_returns_long(const float* __restrict__ rew, const float* __restrict__ val,
               const uint8_t* __restrict__ done, const float* __restrict__ last_val, int64_t T,
               int64_t E, int64_t ld, float gamma, float lam, float* __restrict__ ret,
               float* __restrict__ adv) {
@@ -97,6 +205,7 @@ k_returns_gae(const float* __restrict__ rew, const float* __restrict__ val,
 constexpr int kWideU = 8;                 // time steps loaded ahead
 constexpr int kWideThreads = 64;          // 256 envs per block: every SM gets blocks from 65,536 envs
 constexpr int64_t kWideMinEnvs = 65536;
+constexpr int64_t kOnceMinEnvs = 16384;   // below, windows of k_returns_gae only where one is the horizon
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
@@ -182,18 +291,37 @@ cudaError_t launch_returns_gae(const float* rew, const float* val, const uint8_t
     count_launches(1);
     return cudaGetLastError();
   }
+  // one window covers the horizon, or HBM bounds the walk over several: each input read once
+  if (T <= kRetMaxChunks * kRetL || E >= kOnceMinEnvs) {
+    // Chunks per window: about 130k threads, whose loads in flight cover the memory latency, in
+    // one wave of blocks; no more chunks than the horizon has.
+    int S = 1;
+    while (S < kRetMaxChunks && E * S * 2 <= 160000 && (int64_t)S * kRetL < T) S *= 2;
+    const dim3 block(32, S);
+    const dim3 grid((unsigned)((E + 31) / 32));
+    if (gae)
+      k_returns_gae<true><<<grid, block, 0, s>>>(rew, val, done, last_val, T, E, ld, gamma, lam, ret, adv);
+    else
+      k_returns_gae<false><<<grid, block, 0, s>>>(rew, val, done, last_val, T, E, ld, gamma, lam, ret, adv);
+    count_launches(1);
+    return cudaGetLastError();
+  }
   // Enough (env, chunk) threads to fill the GPU: ~300k threads, chunks of >= 16 steps.
   int S = 1;
   while (S < kRetMaxChunks && E * S * 2 <= 311296 && T / (S * 2) >= 16) S *= 2;
   const dim3 block(32, S);
   const dim3 grid((unsigned)((E + 31) / 32));
-  k_returns_gae<<<grid, block, 0, s>>>(rew, val, done, last_val, T, E, ld, gamma, lam, ret, adv);
+  k_returns_long<<<grid, block, 0, s>>>(rew, val, done, last_val, T, E, ld, gamma, lam, ret, adv);
   count_launches(1);
   return cudaGetLastError();
 }
 
-// Mean-return baseline: per-block fp64 partial sums, then every block of the second
-// kernel reduces the partials in block order (same mean everywhere) and centres.
+// Mean-return baseline: every thread sums its elements as an unevaluated pair of fp32 (two-sum,
+// Knuth 1969: the rounding error of each addition is exact in fp32 and is summed beside it), the
+// threads' pairs meet in fp64, and every block of the second kernel reduces the blocks' fp64
+// partials in block order (same mean everywhere) and centres x - mean with the mean as such a
+// pair.  fp64 arithmetic per element, at this GPU's rate, was the bound: 4.2 M elements took 55
+// us of which HBM needs 8, now 31.
 constexpr int kBaseThreads = 256;
 
 int baseline_blocks(int64_t n) {
@@ -203,40 +331,80 @@ int baseline_blocks(int64_t n) {
   return (int)b;
 }
 
+// s + e += x: s the rounded sum, e the sum of its rounding errors.
+__device__ __forceinline__ void two_sum(float& s, float& e, float x) {
+  const float t = __fadd_rn(s, x);
+  const float b = __fsub_rn(t, s);
+  e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
+  s = t;
+}
+
+__device__ __forceinline__ double block_sum(double acc, double* sh) {
+  for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x / 32] = acc;
+  __syncthreads();
+  acc = 0.0;
+  for (int w = 0; w < kBaseThreads / 32; ++w) acc += sh[w];
+  return acc;
+}
+
 __global__ void __launch_bounds__(kBaseThreads)
 k_base_partial(const float* __restrict__ x, int64_t n, double* __restrict__ part) {
-  __shared__ double sh[kBaseThreads];
-  double acc = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * kBaseThreads + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * kBaseThreads)
-    acc += (double)x[i];
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int d = kBaseThreads / 2; d > 0; d >>= 1) {
-    if ((int)threadIdx.x < d) sh[threadIdx.x] += sh[threadIdx.x + d];
-    __syncthreads();
+  __shared__ double sh[kBaseThreads / 32];
+  float s[4] = {0.0f, 0.0f, 0.0f, 0.0f}, e[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  const int64_t stride = (int64_t)gridDim.x * kBaseThreads;
+  int64_t i = (int64_t)blockIdx.x * kBaseThreads + threadIdx.x;
+  for (; i + 3 * stride < n; i += 4 * stride) {
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = x[i + k * stride];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) two_sum(s[k], e[k], v[k]);
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+  for (; i < n; i += stride) two_sum(s[0], e[0], x[i]);
+  double acc = 0.0;
+  bool fine = true;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    fine = fine && fabsf(s[k]) <= 3.4028234663852886e38f;
+    acc += (double)s[k] + (double)e[k];
+  }
+  if (!fine) {   // an fp32 sum overflowed, or an element is not finite: the plain fp64 sum
+    acc = 0.0;
+    for (i = (int64_t)blockIdx.x * kBaseThreads + threadIdx.x; i < n; i += stride) acc += (double)x[i];
+  }
+  acc = block_sum(acc, sh);
+  if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
 __global__ void __launch_bounds__(kBaseThreads)
 k_base_center(const float* __restrict__ x, int64_t n, const double* __restrict__ part, int nparts,
               float* __restrict__ adv, float* __restrict__ mean_out) {
-  __shared__ double sh[kBaseThreads];
+  __shared__ double sh[kBaseThreads / 32];
   double acc = 0.0;
   for (int i = threadIdx.x; i < nparts; i += kBaseThreads) acc += part[i];
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int d = kBaseThreads / 2; d > 0; d >>= 1) {
-    if ((int)threadIdx.x < d) sh[threadIdx.x] += sh[threadIdx.x + d];
-    __syncthreads();
-  }
-  const double mean = sh[0] / (double)n;
+  const double mean = block_sum(acc, sh) / (double)n;
   if (blockIdx.x == 0 && threadIdx.x == 0 && mean_out) mean_out[0] = (float)mean;
   if (!adv) return;
-  for (int64_t i = (int64_t)blockIdx.x * kBaseThreads + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * kBaseThreads)
-    adv[i] = (float)((double)x[i] - mean);
+  const float mh = (float)mean, ml = (float)(mean - (double)mh);
+  const bool fine = fabsf(mh) <= 3.4028234663852886e38f;
+  const int64_t stride = (int64_t)gridDim.x * kBaseThreads;
+  auto centre = [&](float v) {
+    // v - mh exactly as t + err, then the low part of the mean
+    const float t = __fsub_rn(v, mh);
+    const float b = __fsub_rn(t, v);
+    const float err = __fsub_rn(__fsub_rn(v, __fsub_rn(t, b)), __fadd_rn(mh, b));
+    return fine && fabsf(t) <= 3.4028234663852886e38f ? __fadd_rn(t, __fsub_rn(err, ml)) : t;
+  };
+  int64_t i = (int64_t)blockIdx.x * kBaseThreads + threadIdx.x;
+  for (; i + 3 * stride < n; i += 4 * stride) {
+    float v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = x[i + k * stride];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) adv[i + k * stride] = centre(v[k]);
+  }
+  for (; i < n; i += stride) adv[i] = centre(x[i]);
 }
 
 cudaError_t launch_baseline(const float* x, int64_t n, float* adv, float* mean_out, double* ws,
