@@ -579,8 +579,9 @@ simx_status simx_launch_shape(simx_ctx* c, const simx_mlp* pol, int policy_mode,
     a.bs_pad = a.mlp_warp ? act_stride_pad(a.mlp, 32 / a.G, 32)
                           : act_stride_pad(a.mlp, a.threads / a.G, a.threads);
     plan_rollout(a);
-    host_out[1] = a.G;       // the router's rollout takes its own
+    host_out[1] = a.G;       // the block rollouts take their own
     host_out[2] = a.threads;
+    if (a.fwd.on) host_out[3] = 0;
     host_out[4] = a.tc.on;
     host_out[5] = a.stage.on || a.fwd.on;
   }

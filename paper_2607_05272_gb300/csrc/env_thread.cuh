@@ -53,18 +53,20 @@ __device__ __forceinline__ bool t_count(TScal& s) {
   return false;
 }
 
+// Time of the modulating chain's switch i, given switch i - 1 at t.
+__device__ __forceinline__ uint32_t t_switch_time(const Ctx& x, uint32_t i, uint32_t t, uint32_t& status) {
+  if (x.A.cfg.dwell_kind == 1) return t_add(t, duration_us(x.A.cfg.dwell_mean_us), status);  // a square wave
+  const U4 w = philox(i, x.env, kStreamSwitch, 0u, x.A.key0, x.A.key1);
+  return t_add(t, duration_us(__fmul_rn(x.A.cfg.dwell_mean_us, expo1(w.x))), status);
+}
+
 static __device__ __forceinline__ void t_switches(const Ctx& x, TScal& s, uint32_t limit) {
   if (x.A.cfg.n_mod_states < 2) return;
   while (s.swT <= limit) {
     if (t_count(s)) return;
     s.mst ^= 1u;
     s.swi += 1u;
-    if (x.A.cfg.dwell_kind == 1) {  // fixed dwell: a square wave
-      s.swT = t_add(s.swT, duration_us(x.A.cfg.dwell_mean_us), s.status);
-    } else {
-      const U4 w = philox(s.swi, x.env, kStreamSwitch, 0u, x.A.key0, x.A.key1);
-      s.swT = t_add(s.swT, duration_us(__fmul_rn(x.A.cfg.dwell_mean_us, expo1(w.x))), s.status);
-    }
+    s.swT = t_switch_time(x, s.swi, s.swT, s.status);
   }
 }
 

@@ -90,6 +90,9 @@ cudaError_t launch_rollout(const RolloutArgs& a, cudaStream_t s);
 // rollout_route.cu: the router's rollout with one simulator thread per env
 size_t plan_route(RolloutArgs& a);
 cudaError_t launch_route(const RolloutArgs& a, size_t sh, cudaStream_t s);
+// rollout_single.cu: the same for a single server
+size_t plan_single(RolloutArgs& a);
+cudaError_t launch_single(const RolloutArgs& a, size_t sh, cudaStream_t s);
 // step_thread.cu: one thread per env for the policy-free modes
 bool step_thread_supported(const RolloutArgs& a);
 cudaError_t launch_step_thread(const RolloutArgs& a, cudaStream_t s);
@@ -119,6 +122,8 @@ size_t fwd_plan_biases(const DevMlp& m, FwdPlan& P);
 // Two weight stages from byte `off` on within `budget` bytes of shared memory (at least one row
 // each), and the chunks.
 bool fwd_plan_stages(const DevMlp& m, size_t off, size_t budget, FwdPlan& P);
+// Or the whole policy in shared memory for the launch.
+bool fwd_plan_resident(const DevMlp& m, size_t off, size_t budget, FwdPlan& P);
 size_t fwd_smem(const FwdPlan& P);
 bool plan_policy_block(PolicyArgs& p);
 cudaError_t launch_policy_block(const PolicyArgs& p, cudaStream_t s);

@@ -120,6 +120,24 @@ bool fwd_plan_stages(const DevMlp& m, size_t off, size_t budget, FwdPlan& P) {
   return true;
 }
 
+bool fwd_plan_resident(const DevMlp& m, size_t off, size_t budget, FwdPlan& P) {
+  off = (off + 127) / 128 * 128;
+  P.off = (uint32_t)off;
+  size_t w = 0;
+  P.S = P.n = m.n_layers;
+  for (int l = 0; l < m.n_layers; ++l) {
+    P.woff[l] = (uint32_t)w;
+    w += (size_t)m.dims[l] * m.npad[l + 1] * sizeof(float);   // a multiple of 16 bytes
+    P.rpc[l] = m.dims[l];
+    P.cnt[l] = 1;
+  }
+  if (off + w + 256 > budget) return false;
+  P.bar_off = (uint32_t)(off + (w + 15) / 16 * 16);
+  P.cb = 0;
+  P.resident = 1;
+  return true;
+}
+
 size_t fwd_smem(const FwdPlan& P) { return P.bar_off + fwd::pipe_bytes(P.S); }
 
 // FP32 policies whose layers the register tiles cover; a grid policy's forward rounds between

@@ -141,39 +141,54 @@ __device__ __forceinline__ uint32_t switch_time(const RolloutArgs& A, uint32_t e
   return add_time(t, duration_us(__fmul_rn(A.cfg.dwell_mean_us, expo1(w.x))), status);
 }
 
-// G consecutive candidates from (cand_j, cand_T): lane gl holds candidate cj + gl with
-// its Philox block; times are the prefix sums of integer gaps (exact in any order).  The
+// A chunk of G consecutive candidates, one per lane: lane gl holds candidate base + gl, its time
+// and Philox words.  A chunk stays in registers until every candidate in it is consumed, over as
+// many steps as that takes (a decision consumes from one to some sixty), so that no candidate is
+// drawn twice.
+struct Chunk {
+  uint32_t base, T, wy, wz, ww;
+  bool over;
+};
+
+// The chunk that holds the next candidate (s.cj), drawn if the present one is used up; returns the
+// lane of that candidate.  Times are the prefix sums of integer gaps (exact in any order).  The
 // gap is drawn, or read from entry j mod n of a replayed trace.
 template <int G, bool TR>
-__device__ __forceinline__ void gen_chunk(const RolloutArgs& A, const Grp<G>& g, uint32_t env,
-                                          const Scal& s, uint32_t& T, bool& over, U4& w) {
+__device__ __forceinline__ uint32_t next_chunk(const RolloutArgs& A, const Grp<G>& g, uint32_t env,
+                                               const Scal& s, Chunk& c) {
+  if (s.cj - c.base < (uint32_t)G) return s.cj - c.base;
+  c.base = s.cj;
   const uint32_t j = s.cj + g.gl;
-  w = philox(j, env, kStreamArrival, 0u, A.key0, A.key1);
+  const U4 w = philox(j, env, kStreamArrival, 0u, A.key0, A.key1);
   const uint32_t gap = TR ? A.tr_gap[j % A.tr_n]
                           : duration_us(__fmul_rn(A.cfg.cand_mean_gap_us, expo1(w.x)));
   const uint64_t t64 = (uint64_t)s.cT + g.scan_incl(gap);
-  over = t64 >= kTimeLimit;
-  T = over ? kTimeLimit : (uint32_t)t64;
+  c.over = t64 >= kTimeLimit;
+  c.T = c.over ? kTimeLimit : (uint32_t)t64;
+  c.wy = w.y;
+  c.wz = w.z;
+  c.ww = w.w;
+  return 0u;
 }
 
 // SINGLE mode: consume every candidate with time <= target; accepted ones join
 // their type's FIFO (or are dropped when it is full); switches <= target apply.
 template <int G, bool TR>
-__device__ void advance_single(const RolloutArgs& A, const Grp<G>& g, uint32_t env, Scal& s,
-                               Srv& q, uint32_t* ringb, uint32_t* costb, uint32_t target) {
+__device__ __forceinline__ void advance_single(const RolloutArgs& A, const Grp<G>& g, uint32_t env,
+                                               Scal& s, Srv& q, Chunk& ch, uint32_t* ringb,
+                                               uint32_t* costb, uint32_t target) {
   const simx_config& c = A.cfg;
   const uint32_t cap = c.queue_cap;
   for (;;) {
-    uint32_t T;
-    bool over;
-    U4 w;
-    gen_chunk<G, TR>(A, g, env, s, T, over, w);
-    const bool cons = T <= target;
+    const uint32_t used = next_chunk<G, TR>(A, g, env, s, ch);
+    const uint32_t T = ch.T;
+    const bool cons = g.gl >= used && T <= target;
     const int m = __popc(g.ballot(cons));
-    const int peek = m < G ? m : G - 1;
-    if (g.ballot(over && (int)g.gl <= peek)) s.status |= kStTime;
+    const uint32_t end = used + (uint32_t)m;   // lane of the first candidate left
+    const uint32_t peek = end < (uint32_t)G ? end : (uint32_t)G - 1u;
+    if (g.ballot(ch.over && g.gl >= used && g.gl <= peek)) s.status |= kStTime;
     if (m == 0) break;
-    const uint32_t Tlast = g.shfl(T, m - 1);
+    const uint32_t Tlast = g.shfl(T, (int)end - 1);
     uint32_t st = s.mst;
     if (c.n_mod_states == 2) {
       while (s.swT <= Tlast) {
@@ -187,9 +202,9 @@ __device__ void advance_single(const RolloutArgs& A, const Grp<G>& g, uint32_t e
         }
       }
     }
-    const bool acc = cons && ((w.z >> 8) < c.accept_thr[st]);
-    const uint32_t type = cand_type<TR>(A, s.cj + g.gl, w.y);
-    const uint32_t cst = (acc && (int32_t)type == c.cost_type) ? cand_cost<TR>(A, s.cj + g.gl, w.w) : 0u;
+    const bool acc = cons && ((ch.wz >> 8) < c.accept_thr[st]);
+    const uint32_t type = cand_type<TR>(A, ch.base + g.gl, ch.wy);
+    const uint32_t cst = (acc && (int32_t)type == c.cost_type) ? cand_cost<TR>(A, ch.base + g.gl, ch.ww) : 0u;
     for (uint32_t t = 0; t < c.n_types; ++t) {
       const bool mine = acc && type == t;
       const uint32_t bt = g.ballot(mine);
@@ -218,7 +233,7 @@ __device__ void advance_single(const RolloutArgs& A, const Grp<G>& g, uint32_t e
       s.status |= kStEvent;
       return;
     }
-    if (m < G) break;
+    if (end < (uint32_t)G) break;
   }
   if (c.n_mod_states == 2) {
     while (s.swT <= target) {
@@ -256,63 +271,77 @@ __device__ __forceinline__ void tentative_states(const RolloutArgs& A, uint32_t 
   }
 }
 
-// SINGLE mode: advance to the next accepted arrival and take in all candidates up
-// to its time (the next decision point when nothing is queued).
+// SINGLE mode: the time of the next accepted arrival; rejected candidates before its chunk are
+// consumed.  False when the search gave up (s.status says why).
 template <int G, bool TR>
-__device__ void jump_single(const RolloutArgs& A, const Grp<G>& g, uint32_t env, Scal& s,
-                            Srv& q, uint32_t* ringb, uint32_t* costb) {
+__device__ __forceinline__ bool find_arrival(const RolloutArgs& A, const Grp<G>& g, uint32_t env, Scal& s,
+                                             Chunk& ch, uint32_t& Tf) {
   const simx_config& c = A.cfg;
   for (;;) {
-    uint32_t T;
-    bool over;
-    U4 w;
-    gen_chunk<G, TR>(A, g, env, s, T, over, w);
-    const uint32_t Tmax = g.shfl(T, G - 1);
+    const uint32_t used = next_chunk<G, TR>(A, g, env, s, ch);
+    const uint32_t Tmax = g.shfl(ch.T, G - 1);
     uint32_t st, ms, si, sT, tflag, nsw;
-    tentative_states<G>(A, env, s, T, Tmax, st, ms, si, sT, tflag, nsw);
-    const bool acc = (w.z >> 8) < c.accept_thr[st];
-    const uint32_t bm = g.ballot(acc);
+    tentative_states<G>(A, env, s, ch.T, Tmax, st, ms, si, sT, tflag, nsw);
+    const uint32_t bm = g.ballot(g.gl >= used && (ch.wz >> 8) < c.accept_thr[st]);
     if (bm) {
-      const uint32_t Tf = g.shfl(T, __ffs(bm) - 1);
-      advance_single<G, TR>(A, g, env, s, q, ringb, costb, Tf);
-      s.now = Tf;
-      return;
+      Tf = g.shfl(ch.T, __ffs(bm) - 1);
+      return true;
     }
-    if (g.ballot(over)) s.status |= kStTime;
+    if (g.ballot(ch.over && g.gl >= used)) s.status |= kStTime;
     s.status |= tflag;
     s.mst = ms;
     s.swi = si;
     s.swT = sT;
-    s.cj += G;
+    s.cj += G - used;
     s.cT = Tmax;
-    s.events += G + nsw;
+    s.events += G - used + nsw;
     if (s.events > kEventCap) {
       s.status |= kStEvent;
-      return;
+      return false;
     }
+  }
+}
+
+// SINGLE mode: to the next decision point.  With a batch dispatched (busy), to its end; then, or
+// with nothing queued there, to the next accepted arrival and all candidates up to its time.  One
+// loop, so that the candidate code is in the kernel once (copies of it made instruction fetch a
+// large stall).  A warp of one env (G = 32) keeps its chunk from decision to decision: with the
+// output-per-lane layers and the counted draw (sim.cuh) c1 at 64 envs 5.47 -> 4.53 us per step.
+// Narrower groups begin each decision with a fresh chunk: the extra, partly used one costs them
+// more than drawing its rest again (c2 at 16 lanes: 20.8 against 22.7 us per step).
+template <int G, bool TR>
+__device__ __forceinline__ void to_decision(const RolloutArgs& A, const Grp<G>& g, uint32_t env, Scal& s,
+                                            Srv& q, Chunk& ch, uint32_t* ringb, uint32_t* costb,
+                                            bool busy) {
+  uint32_t target = q.busy;
+  bool arrival = !busy;
+  if (G < 32) ch.base = s.cj - (uint32_t)G;
+  for (;;) {
+    if (arrival && !find_arrival<G, TR>(A, g, env, s, ch, target)) return;
+    advance_single<G, TR>(A, g, env, s, q, ch, ringb, costb, target);
+    s.now = target;
+    if (arrival || q.qc[0] + (A.cfg.n_types > 1 ? q.qc[1] : 0u) != 0u) return;
+    arrival = true;
   }
 }
 
 // ROUTE mode: draw the next request arrival into the pending slot.
 template <int G, bool TR>
-__device__ void next_arrival(const RolloutArgs& A, const Grp<G>& g, uint32_t env, Scal& s) {
+__device__ void next_arrival(const RolloutArgs& A, const Grp<G>& g, uint32_t env, Scal& s, Chunk& ch) {
   const simx_config& c = A.cfg;
   if (TR || c.arrival_kind != SIMX_ARR_DIURNAL) {  // THINNED or TRACE
     for (;;) {
-      uint32_t T;
-      bool over;
-      U4 w;
-      gen_chunk<G, TR>(A, g, env, s, T, over, w);
+      const uint32_t used = next_chunk<G, TR>(A, g, env, s, ch);
+      const uint32_t T = ch.T;
       const uint32_t Tmax = g.shfl(T, G - 1);
       uint32_t st, ms, si, sT, tflag, nsw;
       tentative_states<G>(A, env, s, T, Tmax, st, ms, si, sT, tflag, nsw);
-      const bool acc = (w.z >> 8) < c.accept_thr[st];
-      const uint32_t bm = g.ballot(acc);
+      const uint32_t bm = g.ballot(g.gl >= used && (ch.wz >> 8) < c.accept_thr[st]);
       if (bm) {
         const int f = __ffs(bm) - 1;
         const uint32_t Tf = g.shfl(T, f);
-        const uint32_t wy = g.shfl(w.y, f), ww = g.shfl(w.w, f);
-        if (g.ballot(over && (int)g.gl <= f)) s.status |= kStTime;
+        const uint32_t wy = g.shfl(ch.wy, f), ww = g.shfl(ch.ww, f);
+        if (g.ballot(ch.over && g.gl >= used && (int)g.gl <= f)) s.status |= kStTime;
         if (c.n_mod_states == 2) {
           while (s.swT <= Tf) {
             s.mst ^= 1u;
@@ -324,10 +353,10 @@ __device__ void next_arrival(const RolloutArgs& A, const Grp<G>& g, uint32_t env
             }
           }
         }
-        const uint32_t jf = s.cj + (uint32_t)f;
-        s.cj += (uint32_t)f + 1u;
+        const uint32_t jf = ch.base + (uint32_t)f;
+        s.events += (uint32_t)f - used + 1u;
+        s.cj = jf + 1u;
         s.cT = Tf;
-        s.events += (uint32_t)f + 1u;
         s.pt = Tf;
         s.pty = cand_type<TR>(A, jf, wy);
         s.pc = ((int32_t)s.pty == c.cost_type) ? cand_cost<TR>(A, jf, ww) : 0u;
@@ -335,14 +364,14 @@ __device__ void next_arrival(const RolloutArgs& A, const Grp<G>& g, uint32_t env
         if (s.events > kEventCap) s.status |= kStEvent;
         return;
       }
-      if (g.ballot(over)) s.status |= kStTime;
+      if (g.ballot(ch.over && g.gl >= used)) s.status |= kStTime;
       s.status |= tflag;
       s.mst = ms;
       s.swi = si;
       s.swT = sT;
-      s.cj += G;
+      s.cj += G - used;
       s.cT = Tmax;
-      s.events += G + nsw;
+      s.events += G - used + nsw;
       if (s.events > kEventCap) {
         s.status |= kStEvent;
         return;
@@ -857,6 +886,8 @@ k_rollout(const __grid_constant__ RolloutArgs A) {
   sp.total = (uint32_t)A.H * (uint32_t)A.stage.n;
   if (stg && threadIdx.x == 0) stage_start(A.mlp, A.stage, sp);
 
+  Chunk ch{};
+  ch.base = s.cj - (uint32_t)G;   // nothing drawn yet
   for (int t = 0; t < A.H; ++t) {
     // phase 1: observation (Sec. 4.1) into column `slot` of X0
     if (live) {
@@ -884,7 +915,7 @@ k_rollout(const __grid_constant__ RolloutArgs A) {
                  : mlp_forward_block<GRID>(A.mlp, X0, X1, B, Bs);
       }
       if (live)
-        a = sample_action<G>(A.mlp, Z + slot, Bs, scratch, A.policy_mode, A.key0, A.key1, s.tg,
+        a = sample_action<G, !GRID || G == 32>(A.mlp, Z + slot, Bs, scratch, A.policy_mode, A.key0, A.key1, s.tg,
                              env, logp, value, g);
     } else if (live) {
       a = baseline_action<G, ROUTE>(A, g, env, s, L, ringb);
@@ -937,14 +968,7 @@ k_rollout(const __grid_constant__ RolloutArgs A) {
       __syncwarp();
       if (live && !frozen) {
         s.events = 0;
-        if (n > 0) {
-          const uint32_t next = L.busy;
-          advance_single<G, TR>(A, g, env, s, L, ringb, costb, next);
-          s.now = next;
-          if (L.qc[0] + (T > 1 ? L.qc[1] : 0u) == 0u) jump_single<G, TR>(A, g, env, s, L, ringb, costb);
-        } else {
-          jump_single<G, TR>(A, g, env, s, L, ringb, costb);
-        }
+        to_decision<G, TR>(A, g, env, s, L, ch, ringb, costb, n > 0);
       }
       __syncwarp();
     } else {
@@ -975,7 +999,7 @@ k_rollout(const __grid_constant__ RolloutArgs A) {
       }
       __syncwarp();
       if (live && !frozen) {
-        next_arrival<G, TR>(A, g, env, s);
+        next_arrival<G, TR>(A, g, env, s, ch);
         uint32_t gap = s.pt - now;
         if (gap < 1u) gap = 1u;
         const float inst = __fdiv_rn(1.0e6f, __uint2float_rn(gap));
@@ -1084,12 +1108,14 @@ __global__ void __launch_bounds__(kMaxThreads) k_reset(const __grid_constant__ R
   if (TR)  // this env's starting entry of the trace
     s.cj = (uint32_t)(((uint64_t)w.z * A.tr_n) >> 32);
   Srv L{0u, static_bsize(c), Pair{0u, 0u}, Pair{0u, 0u}};
+  Chunk ch{};
+  ch.base = s.cj - (uint32_t)G;   // nothing drawn yet
   __syncwarp(g.mask);
   if (ROUTE) {
-    next_arrival<G, TR>(A, g, env, s);
+    next_arrival<G, TR>(A, g, env, s, ch);
     s.now = s.pt;
   } else {
-    jump_single<G, TR>(A, g, env, s, L, ringb, costb);
+    to_decision<G, TR>(A, g, env, s, L, ch, ringb, costb, false);
   }
   if (g.gl == 0) store_scal(st, env, s);
   if (ROUTE) {
@@ -1252,7 +1278,7 @@ k_policy_forward(const __grid_constant__ PolicyArgs P) {
   if (!live) return;
   float logp, value;
   const uint32_t env = P.env_base + (uint32_t)i;
-  const int a = sample_action<G>(P.mlp, Z + slot, Bs, scratch, P.mode, P.key0, P.key1, P.step, env,
+  const int a = sample_action<G, true>(P.mlp, Z + slot, Bs, scratch, P.mode, P.key0, P.key1, P.step, env,
                                  logp, value, g);
   if (P.logits)
     for (int j = (int)g.gl; j < P.mlp.n_actions; j += G) P.logits[(int64_t)j * P.ld + i] = Z[j * Bs + slot];
@@ -1439,6 +1465,7 @@ static size_t plan_rollout_t(RolloutArgs& a) {
 
 size_t plan_rollout(RolloutArgs& a) {
   if (const size_t sh = plan_route(a)) return sh;
+  if (const size_t sh = plan_single(a)) return sh;
   const bool route = a.cfg.mode == SIMX_MODE_ROUTE;
   switch (a.G) {
     case 8: return route ? plan_rollout_t<true, 8>(a) : plan_rollout_t<false, 8>(a);
@@ -1491,6 +1518,7 @@ static cudaError_t observe_t(const RolloutArgs& a, cudaStream_t s) {
 cudaError_t launch_rollout(const RolloutArgs& a0, cudaStream_t s) {
   RolloutArgs a = a0;
   if (const size_t sh = plan_route(a)) return launch_route(a, sh, s);
+  if (const size_t sh = plan_single(a)) return launch_single(a, sh, s);
   SIMX_DISPATCH(rollout_t, a, s);
 }
 cudaError_t launch_reset(const RolloutArgs& a, cudaStream_t s) { SIMX_DISPATCH(reset_t, a, s); }

@@ -220,16 +220,6 @@ __device__ __forceinline__ uint32_t* word_ptr(const DevState& st, int w) {
 
 }  // namespace
 
-// The thread's place in the block's virtual order, as a value the compiler cannot carry from
-// one phase of the step to the next: what each phase derives from it (env, columns, pointers)
-// is derived again there, so that none of it is live in the product loops, whose register
-// tiles need the registers.
-__device__ __forceinline__ int place_in_block(int sms) {
-  int t;
-  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
-  return (t + 32 * (int)(blockIdx.x / (unsigned)sms)) & ((int)blockDim.x - 1);
-}
-
 // What a phase derives from the thread's place.
 struct Who {
   int vt, NE, slot, part;
@@ -242,7 +232,7 @@ struct Who {
   __device__ __forceinline__ explicit Who(const RolloutArgs& A, float* smem) {
     const FwdPlan& P = A.fwd;
     unsigned char* sb = reinterpret_cast<unsigned char*>(smem);
-    vt = place_in_block(P.sms);
+    vt = fwd::place_in_block(P.sms);
     NE = 1 << P.ne_shift;
     slot = vt & (NE - 1);
     part = vt >> P.ne_shift;
@@ -271,7 +261,7 @@ __device__ __forceinline__ void phase_observe(const RolloutArgs& A, float* smem,
 template <bool TR>
 __device__ __forceinline__ void phase_ahead(const RolloutArgs& A, float* smem) {
   const FwdPlan& P = A.fwd;
-  const int NE = 1 << P.ne_shift, i = place_in_block(P.sms) - P.side_vt;
+  const int NE = 1 << P.ne_shift, i = fwd::place_in_block(P.sms) - P.side_vt;
   const uint32_t env = blockIdx.x * (uint32_t)NE + (uint32_t)i;
   if (i < 0 || i >= NE || env >= A.st.E) return;
   const Ctx x{A, env, nullptr, nullptr};   // the arrival process reads no ring
@@ -369,7 +359,7 @@ __global__ void __launch_bounds__(NT, MINB) k_route(const __grid_constant__ Roll
   const FwdPlan& P = A.fwd;
   const DevMlp& m = A.mlp;
   const int NE = 1 << P.ne_shift, ld = P.ld;
-  const int vt = place_in_block(P.sms), producer = (int)blockDim.x - 32;
+  const int vt = fwd::place_in_block(P.sms), producer = (int)blockDim.x - 32;
   unsigned char* sb = reinterpret_cast<unsigned char*>(smem);
   const fwd::Pipe p = fwd::pipe_at(sb, P);
   fwd::Place at{0u, 0u};

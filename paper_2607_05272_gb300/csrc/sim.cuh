@@ -89,6 +89,13 @@ struct FwdPlan {
   int side_layer, side_vt;     // layer beside whose products side work runs (-1: none), from thread
   int rpc[SIMX_MAX_LAYERS], cnt[SIMX_MAX_LAYERS];
   int te[SIMX_MAX_LAYERS], to[SIMX_MAX_LAYERS];
+  // resident: the whole policy stays in shared memory for the launch, one chunk per layer (S = n
+  // = the layers), layer l's at byte woff[l] after `off`
+  int resident;
+  uint32_t woff[SIMX_MAX_LAYERS];
+  // rollout_single.cu: byte offsets of the envs' chunks of candidates and of the requests' rings
+  // (0: those stay in global memory)
+  uint32_t win_off, ring_off;
 };
 
 template <int G>
@@ -305,6 +312,25 @@ __device__ __forceinline__ float* mlp_forward_block(const DevMlp& m, float* X0, 
   return in;
 }
 
+// One layer for a single env by one warp: an output per lane (coalesced scalar weights), where
+// 4-output tiles would leave most lanes idle and run four activations one after another.
+template <bool GRID>
+__device__ __forceinline__ void mlp_column(const float* __restrict__ Wt, const float* __restrict__ bias,
+                                           int K, int N, int Npad, const float* x, float* y, int ld, int act,
+                                           int gq, int lane) {
+  for (int j = lane; j < N; j += 32) {
+    float acc = 0.0f;
+    const float* w = Wt + j;
+#pragma unroll 8
+    for (int k = 0; k < K; ++k) acc = __fmaf_rn(__ldg(w + (size_t)k * Npad), x[k * ld], acc);
+    float v = __fadd_rn(acc, __ldg(bias + j));
+    if (act == 0) v = det_tanh(v);
+    else if (act == 2) v = det_gelu(v);
+    if (GRID && gq >= 0) v = grid_q(v, gq);
+    y[j * ld] = v;
+  }
+}
+
 // The same forward for the Bw envs (columns col0 .. col0 + Bw - 1) whose lanes form this
 // warp: only the warp's own lanes take its tiles, so warp barriers replace block
 // barriers.  Every output is still the K-ordered fma chain.  Returns the buffer (not
@@ -324,7 +350,9 @@ __device__ __forceinline__ float* mlp_forward_warp(const DevMlp& m, float* X0, f
     const int K = m.dims[l], N = m.dims[l + 1], Np = m.npad[l + 1];
     const int th = m.act[l];
     const int gq = (GRID && l + 1 < m.n_layers) ? m.gx[l + 1] : -1;
-    if ((Bw / 4) * ((N + 3) / 4) >= 32)
+    if (Bw == 1)
+      mlp_column<GRID>(m.Wt[l], m.bias[l], K, N, Np, in + col0, out + col0, ld, th, gq, lane);
+    else if ((Bw / 4) * ((N + 3) / 4) >= 32)
       mlp_tiles<4, GRID>(m.Wt[l], m.bias[l], K, N, Np, in + col0, out + col0, Bw, ld, th, gq, lane, 32);
     else
       mlp_tiles<1, GRID>(m.Wt[l], m.bias[l], K, N, Np, in + col0, out + col0, Bw, ld, th, gq, lane, 32);
@@ -516,7 +544,9 @@ __device__ __forceinline__ float* mlp_forward_staged(const DevMlp& m, const Stag
 // inversion of the cumulative softmax with a POLICY-stream uniform, ARGMAX takes the
 // first largest logit.  p_i = e^{z_i - max} are computed by the env's lanes in
 // parallel and summed by lane 0 in index order.  logp/value valid in every lane.
-template <int G>
+// COUNT: the draw by counting partial sums, on every lane (c1 at 8000 envs 10.8 -> 10.1 us per
+// step); else by lane 0's search, which left the grid policy's kernel of 8-lane groups 2 % faster.
+template <int G, bool COUNT>
 __device__ __forceinline__ int sample_action(const DevMlp& m, const float* z, int B,
                                              float* scratch, int mode, uint32_t key0,
                                              uint32_t key1, uint32_t step, uint32_t env,
@@ -542,33 +572,67 @@ __device__ __forceinline__ int sample_action(const DevMlp& m, const float* z, in
   }
   for (int i = (int)g.gl; i < A; i += G) scratch[i] = det_exp(__fsub_rn(z[i * B], mx));
   g.sync();
-  int a = 0;
-  float lp = 0.0f;
-  if (g.gl == 0) {
-    float S = 0.0f;
-    for (int i = 0; i < A; ++i) S = __fadd_rn(S, scratch[i]);
-    if (mode == SIMX_POLICY_ARGMAX) {
-      a = ai;
-    } else {
-      const U4 w = philox(step, env, kStreamPolicy, 0u, key0, key1);
-      const float thr = __fmul_rn(u_open1(w.x), S);
-      float cum = 0.0f;
-      a = A - 1;
-      for (int i = 0; i < A; ++i) {
-        cum = __fadd_rn(cum, scratch[i]);
-        if (cum > thr) {
-          a = i;
-          break;
-        }
+  if constexpr (COUNT) {
+    // lane 0 replaces the exponentials by their sums in index order (8 loads before the stores that
+    // might alias them); the draw is then the first sum above u times the last, found by counting
+    // on every lane the sums that are not (they never decrease), else the last action
+    if (g.gl == 0) {
+      float S = 0.0f;
+      for (int i0 = 0; i0 < A; i0 += 8) {
+        float e8[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) e8[i] = i0 + i < A ? scratch[i0 + i] : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (i0 + i < A) {
+            S = __fadd_rn(S, e8[i]);
+            scratch[i0 + i] = S;
+          }
       }
     }
-    lp = __fsub_rn(__fsub_rn(z[a * B], mx), det_log(S));
+    g.sync();
+    const float S = scratch[A - 1];
+    int a = ai < A ? ai : 0;   // (no logit above -inf)
+    if (mode != SIMX_POLICY_ARGMAX) {
+      const U4 w = philox(step, env, kStreamPolicy, 0u, key0, key1);
+      const float thr = __fmul_rn(u_open1(w.x), S);
+      uint32_t cnt = 0u;
+      for (int i = (int)g.gl; i + 1 < A; i += G) cnt += scratch[i] > thr ? 0u : 1u;
+      a = (int)g.sum(cnt);
+    }
+    logp = __fsub_rn(__fsub_rn(z[a * B], mx), det_log(S));
+    value = m.has_value ? z[A * B] : 0.0f;
+    g.sync();
+    return a;
+  } else {
+    int a = 0;
+    float lp = 0.0f;
+    if (g.gl == 0) {
+      float S = 0.0f;
+      for (int i = 0; i < A; ++i) S = __fadd_rn(S, scratch[i]);
+      if (mode == SIMX_POLICY_ARGMAX) {
+        a = ai;
+      } else {
+        const U4 w = philox(step, env, kStreamPolicy, 0u, key0, key1);
+        const float thr = __fmul_rn(u_open1(w.x), S);
+        float cum = 0.0f;
+        a = A - 1;
+        for (int i = 0; i < A; ++i) {
+          cum = __fadd_rn(cum, scratch[i]);
+          if (cum > thr) {
+            a = i;
+            break;
+          }
+        }
+      }
+      lp = __fsub_rn(__fsub_rn(z[a * B], mx), det_log(S));
+    }
+    a = (int)g.shfl((uint32_t)a, 0);
+    logp = g.shflf(lp, 0);
+    value = m.has_value ? z[A * B] : 0.0f;
+    g.sync();
+    return a;
   }
-  a = (int)g.shfl((uint32_t)a, 0);
-  logp = g.shflf(lp, 0);
-  value = m.has_value ? z[A * B] : 0.0f;
-  g.sync();
-  return a;
 }
 
 }  // namespace simx
