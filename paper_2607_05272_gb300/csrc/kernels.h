@@ -112,7 +112,7 @@ struct RepackArgs {
 };
 cudaError_t launch_repack(const RepackArgs& r, cudaStream_t s);
 cudaError_t launch_policy_forward(const PolicyArgs& p, cudaStream_t s);
-// policy_forward.cu: the batched forward of FP32 policies, and the plans that it shares with the
+// policy_forward.cu: the batched forward, and the plans that it shares with the
 // router's rollout.
 // Register tiles of layer l: the largest of 8x8 (big), 4x8, 2x8, 4x4, 2x4, 1x4 that gives `pct`
 // percent of the threads a tile, else the one with the most tiles; also sets P.ne_shift.

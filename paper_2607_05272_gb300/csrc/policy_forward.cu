@@ -1,4 +1,4 @@
-// policy_forward.cu — the batched policy forward (Sec. 4.2) of FP32 policies, and the plans of the
+// policy_forward.cu — the batched policy forward (Sec. 4.2), and the plans of the
 // block forward (fwd_block.cuh) that it shares with the router's rollout.
 //
 // A persistent block takes tiles of NE observation columns: 64 columns on 256 threads with 8x8
@@ -15,7 +15,7 @@
 
 namespace simx {
 
-template <int MINB, bool BIG>
+template <int MINB, bool BIG, bool GRID>
 __global__ void __launch_bounds__(256, MINB) k_forward_block(const __grid_constant__ PolicyArgs A) {
   extern __shared__ __align__(128) float smem[];
   const FwdPlan& P = A.fwd;
@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(256, MINB) k_forward_block(const __grid_consta
     const int64_t col = (tile << P.ne_shift) + slot;
     const bool live = col < A.n;
     for (int d = part; d < D; d += G) smem[d * ld + slot] = live ? __ldg(A.obs + (int64_t)d * A.ld + col) : 0.0f;
-    fwd::forward<BIG>(m, P, p, at, smem, NE, ld, vt, []() {});
+    fwd::forward<BIG, GRID>(m, P, p, at, smem, NE, ld, vt, []() {});
     const float* z = smem + slot;
     if (live && A.logits)
       for (int j = part; j < NA; j += G) A.logits[(int64_t)j * A.ld + col] = z[j * ld];
@@ -140,12 +140,10 @@ bool fwd_plan_resident(const DevMlp& m, size_t off, size_t budget, FwdPlan& P) {
 
 size_t fwd_smem(const FwdPlan& P) { return P.bar_off + fwd::pipe_bytes(P.S); }
 
-// FP32 policies whose layers the register tiles cover; a grid policy's forward rounds between
-// the layers (rollout.cu).
+// Policies (FP32 or grid) whose layers the register tiles cover.
 bool plan_policy_block(PolicyArgs& p) {
   std::memset(&p.fwd, 0, sizeof(p.fwd));
   const DevMlp& m = p.mlp;
-  if (m.grid) return false;
   int maxd = 0;
   for (int l = 0; l <= m.n_layers; ++l) maxd = m.dims[l] > maxd ? m.dims[l] : maxd;
   // columns per block: as many as still give every SM a block
@@ -177,7 +175,8 @@ bool plan_policy_block(PolicyArgs& p) {
 }
 
 cudaError_t launch_policy_block(const PolicyArgs& p, cudaStream_t s) {
-  auto k = p.fwd.big ? k_forward_block<2, true> : k_forward_block<3, false>;
+  auto k = p.mlp.grid ? (p.fwd.big ? k_forward_block<2, true, true> : k_forward_block<3, false, true>)
+                      : (p.fwd.big ? k_forward_block<2, true, false> : k_forward_block<3, false, false>);
   const size_t sh = fwd_smem(p.fwd);
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
   k<<<(unsigned)p.fwd.sms, 256, sh, s>>>(p);

@@ -1254,9 +1254,8 @@ __global__ void __launch_bounds__(256) k_repack(const __grid_constant__ RepackAr
   if (k0 == 0 && ty == 0 && j0 + tx < Np) R.bias[l][j0 + tx] = j0 + tx < N ? R.b[l][j0 + tx] : 0.0f;
 }
 
-// Batched forward (Sec. 4.2) of grid policies, and of FP32 ones whose output layer has too many
-// rows for the register tiles of policy_forward.cu (above 128, off a multiple of 8), over
-// observation columns [D][ld]: a block of B = blockDim.x / G columns runs the block-wide MLP, then each column's G lanes
+// Batched forward (Sec. 4.2) of policies whose output layer has too many rows for the register
+// tiles of policy_forward.cu (above 128, off a multiple of 8), over observation columns [D][ld]: a block of B = blockDim.x / G columns runs the block-wide MLP, then each column's G lanes
 // sample.  Every lane stays alive for the block barriers.
 template <int G>
 __global__ void __launch_bounds__(kMaxThreads)

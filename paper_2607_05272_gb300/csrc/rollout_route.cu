@@ -1,4 +1,4 @@
-// rollout_route.cu — the router's rollout (ROUTE mode, Sec. 3.1, 4.1) with an FP32 policy
+// rollout_route.cu — the router's rollout (ROUTE mode, Sec. 3.1, 4.1) with a policy network
 // whose weights are streamed through shared memory: one thread per env runs the simulator,
 // the whole block runs the policy forward.
 //
@@ -353,7 +353,7 @@ __device__ __forceinline__ void phase_step(const RolloutArgs& A, float* smem, in
   }
 }
 
-template <bool TR, int NT, int MINB, bool BIG>
+template <bool TR, int NT, int MINB, bool BIG, bool GRID>
 __global__ void __launch_bounds__(NT, MINB) k_route(const __grid_constant__ RolloutArgs A) {
   extern __shared__ __align__(128) float smem[];
   const FwdPlan& P = A.fwd;
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(NT, MINB) k_route(const __grid_constant__ Roll
 
   phase_observe(A, smem, 0);
   for (int t = 0; t < A.H; ++t) {
-    fwd::forward<BIG>(m, P, p, at, smem, NE, ld, vt, [&]() { phase_ahead<TR>(A, smem); });
+    fwd::forward<BIG, GRID>(m, P, p, at, smem, NE, ld, vt, [&]() { phase_ahead<TR>(A, smem); });
     phase_step<TR>(A, smem, t);
   }
   __syncthreads();
@@ -406,25 +406,34 @@ __global__ void __launch_bounds__(NT, MINB) k_route(const __grid_constant__ Roll
 
 namespace {
 
+template <bool TR, bool GRID>
+const void* pick_kernel_t(const RolloutArgs& a) {
+  if (a.fwd.big) return (const void*)k_route<TR, 256, 2, true, GRID>;
+  if (a.threads > 128) return (const void*)k_route<TR, 256, 3, false, GRID>;
+  return (const void*)k_route<TR, 128, 7, false, GRID>;
+}
 const void* pick_kernel(const RolloutArgs& a) {
   const bool tr = a.cfg.arrival_kind == SIMX_ARR_TRACE;
-  if (a.fwd.big) return tr ? (const void*)k_route<true, 256, 2, true> : (const void*)k_route<false, 256, 2, true>;
-  if (a.threads > 128) return tr ? (const void*)k_route<true, 256, 3, false> : (const void*)k_route<false, 256, 3, false>;
-  return tr ? (const void*)k_route<true, 128, 7, false> : (const void*)k_route<false, 128, 7, false>;
+  if (a.mlp.grid) return tr ? pick_kernel_t<true, true>(a) : pick_kernel_t<false, true>(a);
+  return tr ? pick_kernel_t<true, false>(a) : pick_kernel_t<false, false>(a);
 }
 
 int r4(int v) { return (v + 3) / 4 * 4; }
 
 }  // namespace
 
-// The plan of k_route for this launch: a.fwd.on when it applies (ROUTE mode, an FP32 policy
-// network of at least kStageMinBytes of weights, or any with SIMX_STAGE=1; SIMX_STAGE=0 turns
+// The plan of k_route for this launch: a.fwd.on when it applies (ROUTE mode, a policy network of at least kStageMinBytes of weights, or any with SIMX_STAGE=1; SIMX_STAGE=0 turns
 // it off), with the shared-memory layout; returns the dynamic shared memory.
 size_t plan_route(RolloutArgs& a) {
   std::memset(&a.fwd, 0, sizeof(a.fwd));
   const DevMlp& m = a.mlp;
   const bool net = a.policy_mode == SIMX_POLICY_SAMPLE || a.policy_mode == SIMX_POLICY_ARGMAX;
-  if (a.cfg.mode != SIMX_MODE_ROUTE || !net || m.grid) return 0;
+  if (a.cfg.mode != SIMX_MODE_ROUTE || !net) return 0;
+  const bool forced = getenv("SIMX_LANES") || getenv("SIMX_THREADS");
+  // A grid policy's forward on the tensor cores (rollout.cu) pays from about 65,536 envs on (c5:
+  // 114 against 121 us per step there; c3 at 16,384 66 against 39, at 1000 46 against 11); it and
+  // its FP32 form are also taken when asked for by their switches.
+  if (m.grid && (forced || getenv("SIMX_TC_FORWARD") || a.st.E > 49152u)) return 0;
   int force = -1;
   if (const char* f = getenv("SIMX_STAGE"))
     if (f[0]) force = f[0] == '0' ? 0 : 1;
@@ -440,7 +449,7 @@ size_t plan_route(RolloutArgs& a) {
   // while that fills the SMs once, then 16, then 32 (the lane-group kernel's choice of 64-thread
   // blocks of 4 or 8 envs ran c4 at 4096 envs in 170 us per step, these in 34)
   int G = a.G, threads = a.threads;
-  if (!getenv("SIMX_LANES") && !getenv("SIMX_THREADS")) {
+  if (!forced) {
     const int64_t E = a.st.E, sms = sm_count();
     if (E <= 14 * sms) {
       threads = 256;

@@ -40,12 +40,14 @@ CASES = [
     ("three-servers-one-type", _router(3, 1, 700), [64, 33], None, "sample", 40),
     ("one-server", _router(1, 2, 300), [40], None, "sample", 40),
     ("five-servers-deep", _router(5, 2, 2500), [31, 64, 17, 128], ["tanh"] * 4, "sample", 24),
+    ("grid-128-threads", W.c3(14701), [128, 128], None, "sample", 16),
+    ("grid-wide", W.c4(2131), [256, 255], ["tanh", "gelu"], "argmax", 16),
     ("trace", W.c3t(900), [128, 128], None, "sample", 40),
 ]
 
 
 @pytest.mark.parametrize("cfg,hidden,acts,mode,H", [c[1:] for c in CASES], ids=[c[0] for c in CASES])
-def test_route_rollout(cfg, hidden, acts, mode, H, monkeypatch):
+def test_route_rollout(cfg, hidden, acts, mode, H, request, monkeypatch):
     from paper_2607_05272_gb300 import build as B
     B.build()
     from paper_2607_05272_gb300 import simx
@@ -54,11 +56,15 @@ def test_route_rollout(cfg, hidden, acts, mode, H, monkeypatch):
     E, dims = cfg["n_envs"], _dims(cfg, hidden)
     Ws, bs = W.mlp_weights(dims, 11, sigma=0.2)
     bs = [b + np.float32(0.05) * np.arange(len(b), dtype=np.float32) / len(b) for b in bs]
+    gx = None
+    if "grid" in request.node.callspec.id:
+        gx, ew = [4] + [7] * len(hidden), [6] * (len(hidden) + 1)
+        Ws, bs = W.grid_weights(dims, 5, gx, ew)
     got = []
     for stage in ("1", "0"):
         monkeypatch.setenv("SIMX_STAGE", stage)
         pol = simx.Policy([torch.from_numpy(w).cuda() for w in Ws],
-                          [torch.from_numpy(b).cuda() for b in bs], True, acts)
+                          [torch.from_numpy(b).cuda() for b in bs], True, acts, grid=gx)
         sim = simx.Sim(cfg)
         sim.reset(0xA11)
         shape = sim.launch_shape(mode, pol)
@@ -76,7 +82,7 @@ def test_route_rollout(cfg, hidden, acts, mode, H, monkeypatch):
         assert torch.equal(a[k], b[k]), k
     assert torch.equal(na, nb) and np.array_equal(sa, sb)
     envs = sorted({0, E // 2, E - 1} | {e for e in (31, 32, 127) if e < E})
-    ref = oracle.rollout(cfg, (Ws, bs, True, acts or ["tanh"] * len(hidden)), 0xA11,
+    ref = oracle.rollout(cfg, (Ws, bs, True, acts or ["tanh"] * len(hidden), gx), 0xA11,
                          {"sample": 0, "argmax": 1}[mode], envs, H)
     sel = torch.tensor(envs, device="cuda")
     col = {k: v.index_select(v.dim() - 1, sel).cpu().numpy() for k, v in a.items()}
