@@ -168,8 +168,22 @@ struct LossArgs {
   int gx[SIMX_MAX_LAYERS];   // grid policy: input grid exponent of layer l
 };
 size_t loss_workspace_bytes(const LossArgs& a);
+// W_l as [K][npad] transposed and [N][kpad] copies, zero padded, every layer in one launch
+struct LossPack {
+  const float* W[SIMX_MAX_LAYERS];
+  float* Wt[SIMX_MAX_LAYERS];
+  float* Wn[SIMX_MAX_LAYERS];
+  int N[SIMX_MAX_LAYERS], K[SIMX_MAX_LAYERS], npad[SIMX_MAX_LAYERS], kpad[SIMX_MAX_LAYERS];
+  int n_layers;
+};
+void launch_pack_loss_w(const LossPack& p, cudaStream_t s);
+// loss_block.cu
+int loss_block_rows(const LossArgs& a);   // rows per block, 0: does not fit
+size_t loss_block_workspace(const LossArgs& a);
+cudaError_t launch_loss_block(const LossArgs& a, void* ws, size_t ws_bytes, cudaStream_t s);
 // loss_fused.cu
 bool loss_fused_fits(const LossArgs& a);
+int64_t loss_fused_rows(const LossArgs& a);   // rows that the busiest block takes
 size_t loss_fused_workspace(const LossArgs& a);
 cudaError_t launch_loss_fused(const LossArgs& a, void* ws, size_t ws_bytes, cudaStream_t s);
 void launch_loss_reduce(const float* part, int nb, int n_params, const double* spart,

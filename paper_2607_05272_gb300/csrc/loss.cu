@@ -369,6 +369,15 @@ static WsLayout layout(const LossArgs& a) {
   return w;
 }
 
+// The block kernel where its one tile per SM has fewer rows than the fused kernel's busiest block
+// walks (5000 rows of 13-128-128-17: 40 against 64; at 4096 both have 32 and the fused one is the
+// faster, 50 us against 53), and only within the scratch that the call has always asked for.
+static bool loss_block_taken(const LossArgs& a) {
+  const int R = loss_block_rows(a);
+  return R > 0 && loss_fused_fits(a) && R < loss_fused_rows(a) &&
+         loss_block_workspace(a) <= loss_fused_workspace(a);
+}
+
 // Large enough for every path, so that the size does not depend on the precision.
 size_t loss_workspace_bytes(const LossArgs& a) {
   const size_t f = loss_fused_fits(a) ? loss_fused_workspace(a) : layout(a).total;
@@ -388,6 +397,7 @@ cudaError_t launch_loss_grad(const LossArgs& a, void* ws, size_t ws_bytes, cudaS
     return loss_fused_fits(a) ? launch_loss_fused(a, ws, ws_bytes, s) : cudaErrorInvalidValue;
   if (a.precision == SIMX_PREC_TF32 && loss_tc_fits(a)) return launch_loss_tc(a, ws, ws_bytes, s);
   if (a.precision == SIMX_PREC_TF32 && loss_wide_fits(a)) return launch_loss_wide(a, ws, ws_bytes, s);
+  if (loss_block_taken(a)) return launch_loss_block(a, ws, ws_bytes, s);
   if (loss_fused_fits(a)) return launch_loss_fused(a, ws, ws_bytes, s);
   const WsLayout w = layout(a);
   if (ws_bytes < w.total) return cudaErrorInvalidValue;

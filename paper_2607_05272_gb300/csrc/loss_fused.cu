@@ -513,14 +513,8 @@ __global__ void __launch_bounds__(kLThreads) k_loss_fused(const __grid_constant_
 
 // Transposed (forward) and row-major padded (backward) copies of each W_l; blockIdx.y
 // is the layer, so one launch packs them all.
-struct PackArgs {
-  const float* W[SIMX_MAX_LAYERS];
-  float* Wt[SIMX_MAX_LAYERS];
-  float* Wn[SIMX_MAX_LAYERS];
-  int N[SIMX_MAX_LAYERS], K[SIMX_MAX_LAYERS], npad[SIMX_MAX_LAYERS], kpad[SIMX_MAX_LAYERS];
-};
-
-__global__ void k_pack_loss_w(const __grid_constant__ PackArgs P) {
+__global__ void k_pack_loss_w(const __grid_constant__ LossPack P) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int l = blockIdx.y;
   const float* __restrict__ W = P.W[l];
   float* __restrict__ Wt = P.Wt[l];
@@ -630,7 +624,22 @@ FusedPlan plan(const LossArgs& a) {
 }
 }  // namespace
 
+void launch_pack_loss_w(const LossPack& p, cudaStream_t s) {
+  int n = 0;
+  for (int l = 0; l < p.n_layers; ++l) {
+    n = p.K[l] * p.npad[l] > n ? p.K[l] * p.npad[l] : n;
+    n = p.N[l] * p.kpad[l] > n ? p.N[l] * p.kpad[l] : n;
+  }
+  k_pack_loss_w<<<dim3((unsigned)((n + 255) / 256), (unsigned)p.n_layers), 256, 0, s>>>(p);
+  count_launches(1);
+}
+
 bool loss_fused_fits(const LossArgs& a) { return plan(a).ok; }
+int64_t loss_fused_rows(const LossArgs& a) {
+  const FusedPlan p = plan(a);
+  const int64_t ntiles = (a.n + p.R - 1) / p.R;
+  return (ntiles + p.grid - 1) / p.grid * p.R;
+}
 size_t loss_fused_workspace(const LossArgs& a) { return plan(a).total; }
 
 cudaError_t launch_loss_fused(const LossArgs& a, void* ws, size_t ws_bytes, cudaStream_t s) {
@@ -639,14 +648,11 @@ cudaError_t launch_loss_fused(const LossArgs& a, void* ws, size_t ws_bytes, cuda
   char* base = static_cast<char*>(ws);
   FusedLossArgs F{};
   F.a = a;
-  PackArgs pk{};
-  int nmax = 0;
+  LossPack pk{};
+  pk.n_layers = a.n_layers;
   for (int l = 0; l < a.n_layers; ++l) {
     float* Wt = reinterpret_cast<float*>(base + p.w_off[l][0]);
     float* Wn = reinterpret_cast<float*>(base + p.w_off[l][1]);
-    const int n = a.dims[l] * p.npad[l + 1] > a.dims[l + 1] * p.kpad[l] ? a.dims[l] * p.npad[l + 1]
-                                                                         : a.dims[l + 1] * p.kpad[l];
-    nmax = n > nmax ? n : nmax;
     pk.W[l] = a.W[l];
     pk.Wt[l] = Wt;
     pk.Wn[l] = Wn;
@@ -657,7 +663,7 @@ cudaError_t launch_loss_fused(const LossArgs& a, void* ws, size_t ws_bytes, cuda
     F.Wt[l] = Wt;
     F.Wn[l] = Wn;
   }
-  k_pack_loss_w<<<dim3((unsigned)((nmax + 255) / 256), (unsigned)a.n_layers), 256, 0, s>>>(pk);
+  launch_pack_loss_w(pk, s);
   for (int l = 0; l <= a.n_layers; ++l) {
     F.npad[l] = p.npad[l];
     F.kpad[l] = p.kpad[l];
@@ -677,7 +683,7 @@ cudaError_t launch_loss_fused(const LossArgs& a, void* ws, size_t ws_bytes, cuda
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
   k<<<p.grid, kLThreads, p.smem, s>>>(F);
   launch_loss_reduce(F.part, p.grid, p.n_params, F.spart, a, s);
-  count_launches(2);
+  count_launches(1);
   return cudaGetLastError();
 }
 
@@ -704,7 +710,15 @@ __global__ void __launch_bounds__(256) k_reduce_all(const float* __restrict__ pa
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P) return;
     float s = 0.0f;
-    for (int b = 0; b < nb; ++b) s += part[(size_t)b * P + i];
+    int b = 0;
+    for (; b + 8 <= nb; b += 8) {   // eight loads in flight, added in order
+      float v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = part[(size_t)(b + q) * P + i];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) s += v[q];
+    }
+    for (; b < nb; ++b) s += part[(size_t)b * P + i];
     out[i] = s;
     return;
   }

@@ -1,0 +1,24 @@
+"""FP32 loss gradient over minibatches of one tile per SM: the block kernel's range and the sizes
+beside it, against the fp64 oracle with the tolerances of the other FP32 paths."""
+import numpy as np
+import pytest
+
+from test_gpu_rl import _check_grad, _loss_case, _simx
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("name,algo,E,H,nmb,hidden", [
+    ("c3", "ppo", 40, 256, 4864, None),         # 32 rows per SM: the fused kernel
+    ("c3", "ppo", 40, 256, 4865, None),         # first of the range: 40-row tiles, the last ragged
+    ("c3", "reinforce", 40, 256, 6081, None),   # 48 rows, the last tile one row
+    ("c3", "ppo", 40, 256, 9728, None),         # last of the range: 64 rows on every SM
+    ("c3", "ppo", 40, 256, 9729, None),         # past it
+    ("c3", "reinforce", 71, 101, None, 100),    # every row, widths off the tiles of 8
+    ("c3s", "ppo", 32, 256, 8192, None),        # two-tower policy
+])
+def test_block_loss_gradient_matches_oracle(name, algo, E, H, nmb, hidden):
+    g, s, g_ref, st, layers, n = _loss_case(_simx(), name, algo, E, H, nmb, "fp32", hidden)
+    _check_grad(g, g_ref, layers)
+    assert np.all(np.abs(s[:4] - st[:4]) <= 1e-5 * (np.abs(st[:4]) + 1.0))
+    assert abs(s[4] - st[4]) <= 1.0 / n
