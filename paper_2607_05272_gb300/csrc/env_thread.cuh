@@ -181,19 +181,27 @@ __device__ __forceinline__ void t_start(const Ctx& x, TScal& s, TSrv& r, int srv
   const uint32_t n = r.bsize < qn ? r.bsize : qn;
   const bool costed = (int32_t)h == c.cost_type;
   uint64_t W = 0, csum = 0;
-  // U requests at a time, their loads in flight together
-  for (uint32_t j = 0; j < n; j += U) {
-    uint32_t tu[U], cu[U];
-#pragma unroll
-    for (uint32_t i = 0; i < U; ++i) {
-      const uint32_t slot = (head + j + i) & (cap - 1u);
-      tu[i] = j + i < n ? rs[h * cap + slot] : st;
-      cu[i] = costed && j + i < n ? x.cost[(size_t)srv * cap + slot] : 0u;
+  if constexpr (U == 1u) {
+    for (uint32_t j = 0; j < n; ++j) {
+      const uint32_t slot = (head + j) & (cap - 1u);
+      W += (uint64_t)(st - rs[h * cap + slot]);
+      if (costed) csum += x.cost[(size_t)srv * cap + slot];
     }
+  } else {
+    // U requests at a time, their loads in flight together
+    for (uint32_t j = 0; j < n; j += U) {
+      uint32_t tu[U], cu[U];
 #pragma unroll
-    for (uint32_t i = 0; i < U; ++i) {
-      W += (uint64_t)(st - tu[i]);
-      csum += cu[i];
+      for (uint32_t i = 0; i < U; ++i) {
+        const uint32_t slot = (head + j + i) & (cap - 1u);
+        tu[i] = j + i < n ? rs[h * cap + slot] : st;
+        cu[i] = costed && j + i < n ? x.cost[(size_t)srv * cap + slot] : 0u;
+      }
+#pragma unroll
+      for (uint32_t i = 0; i < U; ++i) {
+        W += (uint64_t)(st - tu[i]);
+        csum += cu[i];
+      }
     }
   }
   if (h) {

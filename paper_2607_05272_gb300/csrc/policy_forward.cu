@@ -27,14 +27,14 @@ __global__ void __launch_bounds__(256, MINB) k_forward_block(const __grid_consta
   fwd::Place at{0u, 0u};
   const int64_t tiles = (A.n + NE - 1) >> P.ne_shift;
   const int64_t mine = (tiles - blockIdx.x + gridDim.x - 1) / gridDim.x;
-  if (vt == producer) fwd::start(m, P, p, (uint32_t)mine * (uint32_t)P.n);
+  if (vt == producer) fwd::start<false>(m, P, p, (uint32_t)mine * (uint32_t)P.n);
   fwd::load_biases(m, P, p);
   const int D = m.dims[0], NA = m.n_actions;
   for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const int64_t col = (tile << P.ne_shift) + slot;
     const bool live = col < A.n;
     for (int d = part; d < D; d += G) smem[d * ld + slot] = live ? __ldg(A.obs + (int64_t)d * A.ld + col) : 0.0f;
-    fwd::forward<BIG, GRID>(m, P, p, at, smem, NE, ld, vt, []() {});
+    fwd::forward<BIG, GRID, false>(m, P, p, at, smem, NE, ld, vt, []() {});
     const float* z = smem + slot;
     if (live && A.logits)
       for (int j = part; j < NA; j += G) A.logits[(int64_t)j * A.ld + col] = z[j * ld];

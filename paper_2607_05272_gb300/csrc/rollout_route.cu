@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(NT, MINB) k_route(const __grid_constant__ Roll
   unsigned char* sb = reinterpret_cast<unsigned char*>(smem);
   const fwd::Pipe p = fwd::pipe_at(sb, P);
   fwd::Place at{0u, 0u};
-  if (vt == producer) fwd::start(m, P, p, (uint32_t)A.H * (uint32_t)P.n);
+  if (vt == producer) fwd::start<false>(m, P, p, (uint32_t)A.H * (uint32_t)P.n);
   fwd::load_biases(m, P, p);
   {
     const DevState& st = A.st;
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(NT, MINB) k_route(const __grid_constant__ Roll
 
   phase_observe(A, smem, 0);
   for (int t = 0; t < A.H; ++t) {
-    fwd::forward<BIG, GRID>(m, P, p, at, smem, NE, ld, vt, [&]() { phase_ahead<TR>(A, smem); });
+    fwd::forward<BIG, GRID, false>(m, P, p, at, smem, NE, ld, vt, [&]() { phase_ahead<TR>(A, smem); });
     phase_step<TR>(A, smem, t);
   }
   __syncthreads();
@@ -422,8 +422,9 @@ int r4(int v) { return (v + 3) / 4 * 4; }
 
 }  // namespace
 
-// The plan of k_route for this launch: a.fwd.on when it applies (ROUTE mode, a policy network of at least kStageMinBytes of weights, or any with SIMX_STAGE=1; SIMX_STAGE=0 turns
-// it off), with the shared-memory layout; returns the dynamic shared memory.
+// The plan of k_route for this launch: a.fwd.on when it applies (ROUTE mode, a policy network of
+// at least kStageMinBytes of weights, or any with SIMX_STAGE=1; SIMX_STAGE=0 turns it off), with the
+// shared-memory layout; returns the dynamic shared memory.
 size_t plan_route(RolloutArgs& a) {
   std::memset(&a.fwd, 0, sizeof(a.fwd));
   const DevMlp& m = a.mlp;

@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(256, 3) k_single(const __grid_constant__ Rollo
   unsigned char* sb = reinterpret_cast<unsigned char*>(smem);
   const fwd::Pipe p = fwd::pipe_at(sb, P);
   fwd::Place at{0u, 0u};
-  if (vt == producer) fwd::start(m, P, p, P.resident ? (uint32_t)P.n : (uint32_t)A.H * (uint32_t)P.n);
+  if (vt == producer) fwd::start<true>(m, P, p, P.resident ? (uint32_t)P.n : (uint32_t)A.H * (uint32_t)P.n);
   fwd::load_biases(m, P, p);
   uint32_t* words = reinterpret_cast<uint32_t*>(sb + P.st_off);
   const uint32_t env0 = blockIdx.x * (uint32_t)NE;
@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(256, 3) k_single(const __grid_constant__ Rollo
       if (w.vt == 0) *reinterpret_cast<uint32_t*>(sb + P.part_off) = 0u;   // phase_advance's counter
       if (w.part == A.G - 1) w.S[W_U] = philox(w.S[F_TG], w.env, kStreamPolicy, 0u, A.key0, A.key1).x;
     }
-    fwd::forward<false, GRID>(m, P, p, at, smem, NE, ld, vt, []() {});
+    fwd::forward<false, GRID, true>(m, P, p, at, smem, NE, ld, vt, []() {});
     phase_step(A, smem, t);
     __syncthreads();
     phase_advance<TR>(A, smem);
