@@ -371,7 +371,7 @@ static WsLayout layout(const LossArgs& a) {
 
 // The block kernel where its one tile per SM has fewer rows than the fused kernel's busiest block
 // walks (5000 rows of 13-128-128-17: 40 against 64; at 4096 both have 32 and the fused one is the
-// faster, 50 us against 53), and only within the scratch that the call has always asked for.
+// faster, 42 us against 49), and only within the scratch that the call has always asked for.
 static bool loss_block_taken(const LossArgs& a) {
   const int R = loss_block_rows(a);
   return R > 0 && loss_fused_fits(a) && R < loss_fused_rows(a) &&

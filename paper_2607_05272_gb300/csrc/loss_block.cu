@@ -15,10 +15,10 @@
 // What bounds it: latency between barriers (16 warps per SM issue in 36 % of the cycles; the top
 // stalls are shared-memory loads and barriers).  The fused kernel (loss_fused.cu) stages one
 // layer's weights at a time and holds dZ apart, which leaves 8 warps per SM on 32-row tiles: 8192
-// rows of 13-128-128-17 are two rounds of its blocks, 87 us, against one round here, 66 us.  A
-// second tile per block would add to a partial in L2 and measured slower than the fused kernel
-// (65,536 rows: 645 us against 500), as did equal rows per block (4096 rows: 53 against 50), so
-// those stay there.
+// rows of 13-128-128-17 are two rounds of its blocks, 72 us, against one round here, 66 us (4865
+// rows: 70 against 60).  A second tile per block would add to a partial in L2 and measured slower
+// than the fused kernel (65,536 rows: 645 us against 406), as did equal rows per block (4096 rows:
+// 49 against 42), so those stay there.
 #include <cstdint>
 
 #include "fwd_block.cuh"

@@ -11,10 +11,17 @@
 //   db_l += column sums of dZ_l,
 //   dZ_{l-1} = (dZ_l W_l) * (1 - H_l^2).
 // Every GEMM is a register-tiled shared-memory product (4 rows x 4 columns per thread,
-// one float4 of each operand per step).  At the end each block writes its dW/db and
+// one float4 of each operand per step, paired fmas).  At the end each block writes its dW/db and
 // fp64 loss statistics; a second kernel sums the blocks in block order, so the result
 // is deterministic for a given launch configuration.  Nothing touches HBM but the
 // gathered observations and the per-block partials.
+//
+// What bounds it: issue slots and shared-memory latency at 16 (64-row tiles) or 8 warps per SM.
+// Scalar fmas were 40 % of 1295 warp instructions per row of 16-64-64-12, the branching tanh (an
+// IEEE division each) about a fifth: pairs over adjacent outputs (products) or rows (dW: both
+// operands come out of their 16-byte loads as pairs) and the branch-free tanh of the rollouts (the
+// same bits) took 262,144 rows from 546 to 489 us, of 13-128-128-17 from 1877 to 1523 us, and
+// 4096 rows from 46.4 to 39.3 and from 50.0 to 42.5 us.
 //
 // Grid policies (the exact policy forward) run here only: the gathered observations and
 // every hidden output are rounded to their grids exactly as the rollout rounds them, so
@@ -24,7 +31,7 @@
 // layer inputs.
 #include <cstdint>
 
-#include "devmath.cuh"
+#include "fwd_block.cuh"
 #include "kernels.h"
 
 namespace simx {
@@ -65,16 +72,14 @@ __device__ __forceinline__ void tile_gemm_t(const float* __restrict__ Wt, int ld
   const int neb = R / TE, nob = (N + 3) / 4;
   for (int tile = threadIdx.x; tile < neb * nob; tile += blockDim.x) {
     const int eb = tile % neb, ob = tile / neb;
-    float acc[TE][4];
+    uint64_t acc2[TE][2];   // adjacent outputs in pairs
 #pragma unroll
-    for (int e = 0; e < TE; ++e)
-#pragma unroll
-      for (int o = 0; o < 4; ++o) acc[e][o] = 0.0f;
+    for (int e = 0; e < TE; ++e) acc2[e][0] = acc2[e][1] = 0ull;
     const float* wc = Wt + 4 * ob;
     const float* xc = X + TE * eb;
 #pragma unroll 4
     for (int k = 0; k < K; ++k) {
-      const float4 w = *reinterpret_cast<const float4*>(wc + (size_t)k * ldw);
+      const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(wc + (size_t)k * ldw);
       float xv[TE];
       if (TE == 4) {
         const float4 x = *reinterpret_cast<const float4*>(xc + k * kLld);
@@ -87,12 +92,16 @@ __device__ __forceinline__ void tile_gemm_t(const float* __restrict__ Wt, int ld
       }
 #pragma unroll
       for (int e = 0; e < TE; ++e) {
-        acc[e][0] = __fmaf_rn(w.x, xv[e], acc[e][0]);
-        acc[e][1] = __fmaf_rn(w.y, xv[e], acc[e][1]);
-        acc[e][2] = __fmaf_rn(w.z, xv[e], acc[e][2]);
-        acc[e][3] = __fmaf_rn(w.w, xv[e], acc[e][3]);
+        const uint64_t x2 = f2_pack(xv[e], xv[e]);
+        acc2[e][0] = f2_fma(w.x, x2, acc2[e][0]);
+        acc2[e][1] = f2_fma(w.y, x2, acc2[e][1]);
       }
     }
+    float acc[TE][4];
+#pragma unroll
+    for (int e = 0; e < TE; ++e)
+#pragma unroll
+      for (int o = 0; o < 2; ++o) f2_unpack(acc2[e][o], acc[e][2 * o], acc[e][2 * o + 1]);
     if (TE == 4) {
       // the tile's 4 rows of output j are one 16-byte store (conflict-free across
       // the warp's consecutive row blocks)
@@ -128,17 +137,17 @@ __device__ __forceinline__ void tile_gemm_t(const float* __restrict__ Wt, int ld
           const int j = 4 * ob + q / 4;
           if (j < N) grid_act(Y[j * kLld + 4 * eb + q % 4], D[j * kLld + 4 * eb + q % 4], act, gq);
         }
-      } else if (epi == 0 && act == 0) {  // one det_tanh per output, four rows at a time
+      } else if (epi == 0 && act == 0) {  // one output at a time, four rows interleaved
 #pragma unroll 1
         for (int o = 0; o < 4; ++o) {
           const int j = 4 * ob + o;
           if (j < N) {
             float4* y = reinterpret_cast<float4*>(Y + j * kLld + 4 * eb);
             float4 v = *y;
-            v.x = det_tanh(v.x);
-            v.y = det_tanh(v.y);
-            v.z = det_tanh(v.z);
-            v.w = det_tanh(v.w);
+            v.x = fwd::tanh_flat(v.x);
+            v.y = fwd::tanh_flat(v.y);
+            v.z = fwd::tanh_flat(v.z);
+            v.w = fwd::tanh_flat(v.w);
             *y = v;
           }
         }
@@ -179,7 +188,7 @@ __device__ __forceinline__ void tile_gemm_t(const float* __restrict__ Wt, int ld
         for (int o = 0; o < 4; ++o) {
           const int j = 4 * ob + o;
           if (j < N) {
-            if (act == 0) Y[j * kLld + eb] = det_tanh(Y[j * kLld + eb]);
+            if (act == 0) Y[j * kLld + eb] = fwd::tanh_flat(Y[j * kLld + eb]);
             else det_gelu_grad(Y[j * kLld + eb], Y[j * kLld + eb], D[j * kLld + eb]);
           }
         }
@@ -233,30 +242,37 @@ __device__ __forceinline__ void dw_blocks(const float* dz, const float* Hl, int 
   for (int qd = threadIdx.x; qd < nblk * S; qd += blockDim.x) {
     const int blk = qd / S, sp = qd % S;
     const int jb = blk / nk4, kb = blk % nk4;
-    float acc[4][4];
+    uint64_t acc2[4][4];   // sums over the even and the odd rows
 #pragma unroll
     for (int p = 0; p < 4; ++p)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[p][q] = 0.0f;
+      for (int q = 0; q < 4; ++q) acc2[p][q] = 0ull;
 #pragma unroll 2
     for (int r = sp * rs; r < (sp + 1) * rs; r += 4) {
-      float4 dv[4], hv[4];
+      ulonglong2 dv[4], hv[4];
 #pragma unroll
       for (int p = 0; p < 4; ++p) {
         const int j = jb + p * nj4, k = kb + p * nk4;
-        dv[p] = j < N ? *reinterpret_cast<const float4*>(dz + j * kLld + r) : make_float4(0, 0, 0, 0);
-        hv[p] = k < K ? *reinterpret_cast<const float4*>(Hl + k * kLld + r) : make_float4(0, 0, 0, 0);
+        dv[p] = j < N ? *reinterpret_cast<const ulonglong2*>(dz + j * kLld + r) : make_ulonglong2(0, 0);
+        hv[p] = k < K ? *reinterpret_cast<const ulonglong2*>(Hl + k * kLld + r) : make_ulonglong2(0, 0);
       }
 #pragma unroll
       for (int p = 0; p < 4; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          acc[p][q] = __fmaf_rn(dv[p].x, hv[q].x, acc[p][q]);
-          acc[p][q] = __fmaf_rn(dv[p].y, hv[q].y, acc[p][q]);
-          acc[p][q] = __fmaf_rn(dv[p].z, hv[q].z, acc[p][q]);
-          acc[p][q] = __fmaf_rn(dv[p].w, hv[q].w, acc[p][q]);
+          acc2[p][q] = f2_fma(dv[p].x, hv[q].x, acc2[p][q]);
+          acc2[p][q] = f2_fma(dv[p].y, hv[q].y, acc2[p][q]);
         }
     }
+    float acc[4][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float lo, hi;
+        f2_unpack(acc2[p][q], lo, hi);
+        acc[p][q] = lo + hi;
+      }
     if (S > 1) {
       const unsigned gm = split_mask(S);
 #pragma unroll

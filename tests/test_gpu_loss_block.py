@@ -12,8 +12,8 @@ pytestmark = pytest.mark.gpu
     ("c3", "ppo", 40, 256, 4864, None),         # 32 rows per SM: the fused kernel
     ("c3", "ppo", 40, 256, 4865, None),         # first of the range: 40-row tiles, the last ragged
     ("c3", "reinforce", 40, 256, 6081, None),   # 48 rows, the last tile one row
-    ("c3", "ppo", 40, 256, 9728, None),         # last of the range: 64 rows on every SM
-    ("c3", "ppo", 40, 256, 9729, None),         # past it
+    ("c3", "ppo", 40, 256, 8512, None),         # last of the range: 56 rows on every SM
+    ("c3", "ppo", 40, 256, 8513, None),         # past it: 64 rows on either kernel
     ("c3", "reinforce", 71, 101, None, 100),    # every row, widths off the tiles of 8
     ("c3s", "ppo", 32, 256, 8192, None),        # two-tower policy
 ])
