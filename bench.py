@@ -409,12 +409,12 @@ class Clocks:
                 "reasons": reasons, "samples": len(rows)}
 
 
-# DRAM bytes (read + write) of one k_rollout launch of the benchmark workload, from an
+# DRAM bytes (read + write) of one k_route launch of the benchmark workload, from an
 # ncu capture of the current kernel; None until one is taken, and to be re-measured (or
 # set back to None) whenever the rollout kernel changes.
-ROLLOUT_DRAM_BYTES = 389046528.0 + 4584373504.0
-ROLLOUT_DRAM_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_rollout launch "
-                       "of this workload (389.0 MB + 4584.4 MB; profiles/k_rollout_c4_bench.md)")
+ROLLOUT_DRAM_BYTES = 407104512.0 + 4509971968.0
+ROLLOUT_DRAM_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_route launch "
+                       "of this workload (407.1 MB + 4510.0 MB; profiles/k_route_c4_bench.md)")
 
 
 def _peaks():
@@ -961,18 +961,18 @@ def run_gpu(a) -> None:
                      "peak": fp32_nominal, "unit": "TFLOP/s", "frac": ach_l / fp32_nominal,
                      "traffic": None, "peak_source": fp32_src, "ms_per_call": loss_live_ms}
     ach_r = flop_rollout / (ph[1] * 1e-3) / 1e12
-    roof_rollout = {"kernel": "k_rollout (simulation + fused policy)", "bound": "alu",
+    roof_rollout = {"kernel": "k_route (simulation + fused policy)", "bound": "alu",
                     "achieved": ach_r, "peak": fp32_nominal, "unit": "TFLOP/s",
                     "frac": ach_r / fp32_nominal, "traffic": ROLLOUT_DRAM_BYTES,
                     "traffic_source": ROLLOUT_DRAM_SOURCE, "peak_source": fp32_src,
                     "flop_per_launch": flop_rollout}
     # the dominant single kernel: the loss-gradient call is five kernels (weight images,
     # per-tile forward/backward, weight-gradient products, two reductions), the largest
-    # about two thirds of the call (profiles/), so k_rollout leads unless the whole call
+    # about two thirds of the call (profiles/), so the rollout leads unless the whole call
     # outweighs it by more than that
     loss_total_ms = update_ms * loss_share
     roof = roof_rollout if ph[1] >= 0.7 * loss_total_ms else roof_loss
-    roof_rollout["dominance"] = ("k_rollout %.1f ms per step; the loss-gradient calls %.1f ms per "
+    roof_rollout["dominance"] = ("k_route %.1f ms per step; the loss-gradient calls %.1f ms per "
                                  "step over five kernels" % (ph[1], loss_total_ms))
 
     if rank == 0:

@@ -314,12 +314,12 @@ simx_status rollout_collect(simx_ctx* ctx, const simx_mlp* pol, int policy_mode,
  * count).  host_out[6] receives: [0] kernel, 0 = the fused step with the policy forward
  * (one group of lanes per env), 1 = the thread-per-env step of the policy-free modes;
  * [1] lanes per env (1 for the thread-per-env step; the block's threads per env in the
- * router's rollout of an FP32 policy, one of which runs the simulator); [2] threads per block; [3] 1 when
+ * block-wide rollouts, one of which runs the simulator); [2] threads per block; [3] 1 when
  * each warp runs the policy forward for its own envs, 0 for the block-wide forward;
  * [4] 1 when a grid policy's forward runs on the tensor cores (tcgen05, bf16 operands
  * exact on the grid, FP32 accumulation: the FP32 path's bits), 0 otherwise; [5] 1 when
- * the block-wide FP32 forward streams its weights through shared memory (bulk copies
- * into two stages; the same fma chains and bits), 0 otherwise.
+ * the block-wide FP32 forward reads its weights from shared memory (bulk copies, into
+ * stages or once; the same fma chains and bits), 0 otherwise.
  * It exists so that tests and benchmarks can state which instantiation they exercise.
  * SIMX_EINVAL for a NULL argument, an unknown mode or a policy that rollout_collect
  * would refuse.
