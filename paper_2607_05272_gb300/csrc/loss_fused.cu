@@ -20,7 +20,8 @@
 // Scalar fmas were 40 % of 1295 warp instructions per row of 16-64-64-12, the branching tanh (an
 // IEEE division each) about a fifth: pairs over adjacent outputs (products) or rows (dW: both
 // operands come out of their 16-byte loads as pairs) and the branch-free tanh of the rollouts (the
-// same bits) took 262,144 rows from 546 to 489 us, of 13-128-128-17 from 1877 to 1523 us, and
+// same bits) took 262,144 rows from 546 to 489 us (408 with the weights
+// resident, below), of 13-128-128-17 from 1877 to 1523 us, and
 // 4096 rows from 46.4 to 39.3 and from 50.0 to 42.5 us.
 //
 // Grid policies (the exact policy forward) run here only: the gathered observations and
@@ -310,6 +311,7 @@ struct FusedLossArgs {
   int poff[SIMX_MAX_LAYERS];         // offset of layer l's dW in the flat gradient
   int n_params;
   int wst_off;                       // float offset of the weight staging buffer (WS kernels)
+  int wt_off[SIMX_MAX_LAYERS], wn_off[SIMX_MAX_LAYERS];  // floats past it (all weights resident)
   float* part;                       // [gridDim.x][n_params]
   double* spart;                     // [gridDim.x][4]
   int64_t ntiles;
@@ -329,10 +331,13 @@ __device__ __forceinline__ void stage_weights(float* dst, const float* __restric
 
 __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// WS: each layer's weights are staged in shared memory before its product (policies
-// whose weights do not stay in L1 beside one block's shared memory); the products read
-// the same values in the same order either way.
-template <int R, bool WS>
+// WS 1: each layer's weights are staged in shared memory before its product (policies
+// whose weights do not stay in L1 beside one block's shared memory).  WS 2: every weight,
+// in both orders, stays in shared memory, in the place of the dZ buffers: dZ of a hidden
+// layer is written over its activations.  Through what two blocks leave of L1, the
+// 43 KB of 16-64-64-12 missed on every pass (its largest stall): 4096 rows 39.3 -> 31.9 us,
+// 262,144 rows 489 -> 408.  The products read the same values in the same order each way.
+template <int R, int WS>
 __global__ void __launch_bounds__(kLThreads) k_loss_fused(const __grid_constant__ FusedLossArgs F) {
   constexpr int kLR = R, kLld = R + 4, kLanes = kLThreads / R;  // lanes per row in the head
   extern __shared__ float sm[];
@@ -341,8 +346,13 @@ __global__ void __launch_bounds__(kLThreads) k_loss_fused(const __grid_constant_
   float* acts = sm;                                        // all layers' activations
   float* dzA = acts + (size_t)F.act_off[L + 1] * kLld;     // two dZ buffers
   float* dzB = dzA + (size_t)F.dz_rows * kLld;
-  float* gacc = dzB + (size_t)F.dz_rows * kLld;            // dW/db accumulators [n_params]
-  float* wst = sm + F.wst_off;                             // WS: one layer's weights
+  float* gacc = (WS == 2 ? dzA : dzB) + (size_t)F.dz_rows * kLld;  // dW/db accumulators [n_params]
+  float* wst = sm + F.wst_off;                             // WS: one layer's weights, or all
+  if (WS == 2)
+    for (int l = 0; l < L; ++l) {
+      stage_weights(wst + F.wt_off[l], F.Wt[l], a.dims[l] * F.npad[l + 1]);
+      if (l > 0) stage_weights(wst + F.wn_off[l], F.Wn[l], a.dims[l + 1] * F.kpad[l]);
+    }
   for (int i = threadIdx.x; i < F.n_params; i += blockDim.x) gacc[i] = 0.0f;
   double st_pg = 0.0, st_v = 0.0, st_h = 0.0, st_cf = 0.0;
   const int D = a.dims[0];
@@ -352,7 +362,7 @@ __global__ void __launch_bounds__(kLThreads) k_loss_fused(const __grid_constant_
   for (int64_t tile = blockIdx.x; tile < F.ntiles; tile += gridDim.x) {
     const int64_t r0 = tile * kLR;
     __syncthreads();
-    if (WS) stage_weights(wst, F.Wt[0], a.dims[0] * F.npad[1]);  // lands during the gather
+    if (WS == 1) stage_weights(wst, F.Wt[0], a.dims[0] * F.npad[1]);  // lands during the gather
     // gather X [D][R]: thread (r, dq) reads features dq, dq + kLanes, ... of row r
     // (rows past n are zero and have zero dZ); consecutive threads take consecutive
     // rows, so for a fixed feature the reads are coalesced along the env axis
@@ -372,10 +382,11 @@ __global__ void __launch_bounds__(kLThreads) k_loss_fused(const __grid_constant_
         for (int d = dq; d < D; d += kLanes) X[d * kLld + r] = 0.0f;
       }
     }
+    if (WS == 2) stage_wait();
     __syncthreads();
     for (int l = 0; l < L; ++l) {
-      const float* Wf = F.Wt[l];
-      if (WS) {
+      const float* Wf = WS == 2 ? wst + F.wt_off[l] : F.Wt[l];
+      if (WS == 1) {
         if (l > 0) stage_weights(wst, F.Wt[l], a.dims[l] * F.npad[l + 1]);
         stage_wait();
         __syncthreads();
@@ -461,7 +472,7 @@ __global__ void __launch_bounds__(kLThreads) k_loss_fused(const __grid_constant_
       const float* Hl = acts + (size_t)F.act_off[l] * kLld;
       float* gW = gacc + F.poff[l];
       float* gb = gW + (size_t)N * K;
-      if (WS && l > 0) stage_weights(wst, F.Wn[l], N * F.kpad[l]);  // lands during dW, db
+      if (WS == 1 && l > 0) stage_weights(wst, F.Wn[l], N * F.kpad[l]);  // lands during dW, db
       // dW += dZ^T H: 4 x 4 blocks of (j, k); the tile's rows are split over S
       // adjacent lanes (S > 1 for thin layers) whose partial sums are combined before
       // the block's accumulator is updated
@@ -491,15 +502,13 @@ __global__ void __launch_bounds__(kLThreads) k_loss_fused(const __grid_constant_
         }
       }
       if (l > 0) {
-        float* dzn = (dz == dzA) ? dzB : dzA;
+        float* dzn = WS == 2 ? acts + (size_t)F.act_off[l] * kLld : (dz == dzA) ? dzB : dzA;
         // dZ_{l-1}[k][r] = sum_j W_l[j][k] dZ_l[j][r] * (1 - H_l[k][r]^2); grid policies
         // (and GELU layers) multiply by the stored derivative instead
         const int pa = a.grid ? 2 : a.act[l - 1];  // activation whose derivative applies
-        if (WS) {
-          stage_wait();
-          __syncthreads();
-        }
-        tile_gemm<R>(WS ? wst : F.Wn[l], F.kpad[l], N, K, dz, dzn, 1, nullptr, pa,
+        if (WS == 1) stage_wait();
+        if (WS) __syncthreads();   // the weights landed; dW has read the activations
+        tile_gemm<R>(WS == 2 ? wst + F.wn_off[l] : WS ? wst : F.Wn[l], F.kpad[l], N, K, dz, dzn, 1, nullptr, pa,
                      pa == 2 ? acts + (size_t)F.dact_off[l] * kLld : Hl, nullptr);
         __syncthreads();
         dz = dzn;
@@ -554,8 +563,8 @@ struct FusedPlan {
   int npad[SIMX_MAX_LAYERS + 1], kpad[SIMX_MAX_LAYERS + 1], act_off[SIMX_MAX_LAYERS + 2];
   int dact_off[SIMX_MAX_LAYERS + 1];
   int dz_rows, poff[SIMX_MAX_LAYERS], n_params, grid;
-  bool stage;
-  int wst_off;
+  bool stage, resident;
+  int wst_off, wt_off[SIMX_MAX_LAYERS], wn_off[SIMX_MAX_LAYERS];
   size_t smem, w_off[SIMX_MAX_LAYERS][2], part_off, spart_off, total;
 };
 
@@ -613,13 +622,35 @@ FusedPlan plan_r(const LossArgs& a, int R) {
   return p;
 }
 
-// 64-row tiles when two blocks of them fit in shared memory, else 32-row tiles.  A
+// 64-row tiles when two blocks of them fit in shared memory (with every weight resident
+// where dZ over the activations leaves the room), else 32-row tiles.  A
 // plan with one block per SM stages each layer's weights in shared memory when the
 // largest layer fits beside it (then the weights no longer compete with the block's
 // shared memory for L1, where they missed on 128-wide layers).
 FusedPlan plan(const LossArgs& a) {
-  const FusedPlan p64 = plan_r(a, 64);
-  if (p64.ok && p64.smem <= 110 * 1024) return p64;
+  FusedPlan p64 = plan_r(a, 64);
+  if (p64.ok && p64.smem <= 110 * 1024) {
+    bool plain = !a.grid;   // no stored derivatives
+    for (int l = 0; l + 1 < a.n_layers; ++l) plain = plain && a.act[l] != 2;
+    if (!plain) return p64;
+    const int dz_rows = r4(a.dims[a.n_layers]);
+    size_t off = (size_t)(p64.act_off[a.n_layers + 1] + dz_rows) * (64 + 4) + r4(p64.n_params);
+    const int wst = (int)off;
+    for (int l = 0; l < a.n_layers; ++l) {
+      p64.wt_off[l] = (int)off - wst;
+      off += (size_t)a.dims[l] * p64.npad[l + 1];
+      p64.wn_off[l] = (int)off - wst;
+      if (l > 0) off += (size_t)a.dims[l + 1] * p64.kpad[l];
+    }
+    // two blocks per SM: 113 KB each, the static statistics (2 KB) among it
+    if (off * sizeof(float) + 2048 <= 113 * 1024) {
+      p64.resident = true;
+      p64.dz_rows = dz_rows;
+      p64.wst_off = wst;
+      p64.smem = off * sizeof(float);
+    }
+    return p64;
+  }
   FusedPlan p = plan_r(a, 32);
   if (!p.ok || p.smem <= 110 * 1024) return p;
   int wmax = 0;
@@ -694,8 +725,12 @@ cudaError_t launch_loss_fused(const LossArgs& a, void* ws, size_t ws_bytes, cuda
   F.part = reinterpret_cast<float*>(base + p.part_off);
   F.spart = reinterpret_cast<double*>(base + p.spart_off);
   F.ntiles = (a.n + p.R - 1) / p.R;
-  auto k = p.R == 64 ? k_loss_fused<64, false>
-                     : (p.stage ? k_loss_fused<32, true> : k_loss_fused<32, false>);
+  for (int l = 0; l < a.n_layers; ++l) {
+    F.wt_off[l] = p.wt_off[l];
+    F.wn_off[l] = p.wn_off[l];
+  }
+  auto k = p.R == 64 ? (p.resident ? k_loss_fused<64, 2> : k_loss_fused<64, 0>)
+                     : (p.stage ? k_loss_fused<32, 1> : k_loss_fused<32, 0>);
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
   k<<<p.grid, kLThreads, p.smem, s>>>(F);
   launch_loss_reduce(F.part, p.grid, p.n_params, F.spart, a, s);

@@ -22,3 +22,20 @@ def test_block_loss_gradient_matches_oracle(name, algo, E, H, nmb, hidden):
     _check_grad(g, g_ref, layers)
     assert np.all(np.abs(s[:4] - st[:4]) <= 1e-5 * (np.abs(st[:4]) + 1.0))
     assert abs(s[4] - st[4]) <= 1.0 / n
+
+
+@pytest.mark.parametrize("name,algo,E,H,nmb,hidden", [
+    ("c2", "reinforce", 1, 1, None, None),      # one row
+    ("c2", "ppo", 16, 64, 64, None),            # one full tile
+    ("c2", "ppo", 16, 64, 65, None),
+    ("c2", "reinforce", 40, 512, 19457, None),  # one block walks two tiles
+    ("c2", "ppo", 16, 64, 333, 60),             # widths off the tiles
+    ("c2", "ppo", 16, 64, 333, 68),             # the weights no longer fit beside two blocks
+    ("c1", "ppo", 64, 400, 20000, None),
+])
+def test_resident_weights_loss_gradient_matches_oracle(name, algo, E, H, nmb, hidden):
+    """The fused kernel with every weight in shared memory, dZ over the activations."""
+    g, s, g_ref, st, layers, n = _loss_case(_simx(), name, algo, E, H, nmb, "fp32", hidden)
+    _check_grad(g, g_ref, layers)
+    assert np.all(np.abs(s[:4] - st[:4]) <= 1e-5 * (np.abs(st[:4]) + 1.0))
+    assert abs(s[4] - st[4]) <= 1.0 / n
