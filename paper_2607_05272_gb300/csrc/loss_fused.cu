@@ -23,6 +23,8 @@
 // same bits) took 262,144 rows from 546 to 489 us (408 with the weights
 // resident, below), of 13-128-128-17 from 1877 to 1523 us, and
 // 4096 rows from 46.4 to 39.3 and from 50.0 to 42.5 us.
+// The gradient's error against fp64 is 0.95 (c1's policy), 0.98 (c2's) and 0.99 (c3's) of the scalar
+// form's, geometric means over 15 minibatches each.
 //
 // Grid policies (the exact policy forward) run here only: the gathered observations and
 // every hidden output are rounded to their grids exactly as the rollout rounds them, so
