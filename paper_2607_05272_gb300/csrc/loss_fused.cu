@@ -17,14 +17,11 @@
 // gathered observations and the per-block partials.
 //
 // What bounds it: issue slots and shared-memory latency at 16 (64-row tiles) or 8 warps per SM.
-// Scalar fmas were 40 % of 1295 warp instructions per row of 16-64-64-12, the branching tanh (an
-// IEEE division each) about a fifth: pairs over adjacent outputs (products) or rows (dW: both
-// operands come out of their 16-byte loads as pairs) and the branch-free tanh of the rollouts (the
-// same bits) took 262,144 rows from 546 to 489 us (408 with the weights
-// resident, below), of 13-128-128-17 from 1877 to 1523 us, and
-// 4096 rows from 46.4 to 39.3 and from 50.0 to 42.5 us.
-// The gradient's error against fp64 is 0.95 (c1's policy), 0.98 (c2's) and 0.99 (c3's) of the scalar
-// form's, geometric means over 15 minibatches each.
+// The products' paired fmas (over adjacent outputs; each output keeps its k-ordered chain), the
+// branch-free tanh of the rollouts (the same bits; the branching one has an IEEE division each) and
+// for small policies the weights resident in shared memory (below) took 262,144 rows of
+// 16-64-64-12 from 548 to 411 us and of 13-128-128-17 from 1880 to 1571 us, 4096 rows from 46.0 to
+// 32.3 and from 50.2 to 43.3 us, all with the bits of the scalar form.
 //
 // Grid policies (the exact policy forward) run here only: the gathered observations and
 // every hidden output are rounded to their grids exactly as the rollout rounds them, so
@@ -234,8 +231,10 @@ __device__ __forceinline__ unsigned split_mask(int S) {
 // nk4 = ceil(K/4)): neighbouring lanes read neighbouring features, whose rows sit
 // R + 4 floats apart, so a warp's 16-byte row loads are free of bank conflicts.
 // Each block is handled by S adjacent lanes, lane sp summing rows
-// [sp R / S, (sp + 1) R / S); the S partial sums are combined by a fixed xor
-// butterfly, so the order is the same on every run.
+// [sp R / S, (sp + 1) R / S) in order; the S partial sums are combined by a fixed xor
+// butterfly, so the order is the same on every run.  Scalar fmas: pairs would sum the even and
+// the odd rows apart, and a last bit of the first update is enough for the policy to sample
+// another action somewhere among the next iteration's millions.
 template <int R, int S>
 __device__ __forceinline__ void dw_blocks(const float* dz, const float* Hl, int N, int K,
                                           float* gW) {
@@ -245,37 +244,30 @@ __device__ __forceinline__ void dw_blocks(const float* dz, const float* Hl, int 
   for (int qd = threadIdx.x; qd < nblk * S; qd += blockDim.x) {
     const int blk = qd / S, sp = qd % S;
     const int jb = blk / nk4, kb = blk % nk4;
-    uint64_t acc2[4][4];   // sums over the even and the odd rows
+    float acc[4][4];
 #pragma unroll
     for (int p = 0; p < 4; ++p)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc2[p][q] = 0ull;
+      for (int q = 0; q < 4; ++q) acc[p][q] = 0.0f;
 #pragma unroll 2
     for (int r = sp * rs; r < (sp + 1) * rs; r += 4) {
-      ulonglong2 dv[4], hv[4];
+      float4 dv[4], hv[4];
 #pragma unroll
       for (int p = 0; p < 4; ++p) {
         const int j = jb + p * nj4, k = kb + p * nk4;
-        dv[p] = j < N ? *reinterpret_cast<const ulonglong2*>(dz + j * kLld + r) : make_ulonglong2(0, 0);
-        hv[p] = k < K ? *reinterpret_cast<const ulonglong2*>(Hl + k * kLld + r) : make_ulonglong2(0, 0);
+        dv[p] = j < N ? *reinterpret_cast<const float4*>(dz + j * kLld + r) : make_float4(0, 0, 0, 0);
+        hv[p] = k < K ? *reinterpret_cast<const float4*>(Hl + k * kLld + r) : make_float4(0, 0, 0, 0);
       }
 #pragma unroll
       for (int p = 0; p < 4; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          acc2[p][q] = f2_fma(dv[p].x, hv[q].x, acc2[p][q]);
-          acc2[p][q] = f2_fma(dv[p].y, hv[q].y, acc2[p][q]);
+          acc[p][q] = __fmaf_rn(dv[p].x, hv[q].x, acc[p][q]);
+          acc[p][q] = __fmaf_rn(dv[p].y, hv[q].y, acc[p][q]);
+          acc[p][q] = __fmaf_rn(dv[p].z, hv[q].z, acc[p][q]);
+          acc[p][q] = __fmaf_rn(dv[p].w, hv[q].w, acc[p][q]);
         }
     }
-    float acc[4][4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float lo, hi;
-        f2_unpack(acc2[p][q], lo, hi);
-        acc[p][q] = lo + hi;
-      }
     if (S > 1) {
       const unsigned gm = split_mask(S);
 #pragma unroll
