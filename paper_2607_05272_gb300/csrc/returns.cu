@@ -316,12 +316,10 @@ cudaError_t launch_returns_gae(const float* rew, const float* val, const uint8_t
   return cudaGetLastError();
 }
 
-// Mean-return baseline: every thread sums its elements as an unevaluated pair of fp32 (two-sum,
-// Knuth 1969: the rounding error of each addition is exact in fp32 and is summed beside it), the
-// threads' pairs meet in fp64, and every block of the second kernel reduces the blocks' fp64
-// partials in block order (same mean everywhere) and centres x - mean with the mean as such a
-// pair.  fp64 arithmetic per element, at this GPU's rate, was the bound: 4.2 M elements took 55
-// us of which HBM needs 8, now 31.
+// Mean-return baseline: per-block fp64 partial sums, then every block of the second
+// kernel reduces the partials in block order (same mean everywhere) and centres.  fp64
+// arithmetic per element, at this GPU's rate, is the bound; sums as pairs of fp32, whose low
+// words lose bits where the elements cancel, would take about half the time and are not used.
 constexpr int kBaseThreads = 256;
 
 int baseline_blocks(int64_t n) {
@@ -331,80 +329,40 @@ int baseline_blocks(int64_t n) {
   return (int)b;
 }
 
-// s + e += x: s the rounded sum, e the sum of its rounding errors.
-__device__ __forceinline__ void two_sum(float& s, float& e, float x) {
-  const float t = __fadd_rn(s, x);
-  const float b = __fsub_rn(t, s);
-  e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
-  s = t;
-}
-
-__device__ __forceinline__ double block_sum(double acc, double* sh) {
-  for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x / 32] = acc;
-  __syncthreads();
-  acc = 0.0;
-  for (int w = 0; w < kBaseThreads / 32; ++w) acc += sh[w];
-  return acc;
-}
-
 __global__ void __launch_bounds__(kBaseThreads)
 k_base_partial(const float* __restrict__ x, int64_t n, double* __restrict__ part) {
-  __shared__ double sh[kBaseThreads / 32];
-  float s[4] = {0.0f, 0.0f, 0.0f, 0.0f}, e[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  const int64_t stride = (int64_t)gridDim.x * kBaseThreads;
-  int64_t i = (int64_t)blockIdx.x * kBaseThreads + threadIdx.x;
-  for (; i + 3 * stride < n; i += 4 * stride) {
-    float v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = x[i + k * stride];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) two_sum(s[k], e[k], v[k]);
-  }
-  for (; i < n; i += stride) two_sum(s[0], e[0], x[i]);
+  __shared__ double sh[kBaseThreads];
   double acc = 0.0;
-  bool fine = true;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    fine = fine && fabsf(s[k]) <= 3.4028234663852886e38f;
-    acc += (double)s[k] + (double)e[k];
+  for (int64_t i = (int64_t)blockIdx.x * kBaseThreads + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * kBaseThreads)
+    acc += (double)x[i];
+  sh[threadIdx.x] = acc;
+  __syncthreads();
+  for (int d = kBaseThreads / 2; d > 0; d >>= 1) {
+    if ((int)threadIdx.x < d) sh[threadIdx.x] += sh[threadIdx.x + d];
+    __syncthreads();
   }
-  if (!fine) {   // an fp32 sum overflowed, or an element is not finite: the plain fp64 sum
-    acc = 0.0;
-    for (i = (int64_t)blockIdx.x * kBaseThreads + threadIdx.x; i < n; i += stride) acc += (double)x[i];
-  }
-  acc = block_sum(acc, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = acc;
+  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
 __global__ void __launch_bounds__(kBaseThreads)
 k_base_center(const float* __restrict__ x, int64_t n, const double* __restrict__ part, int nparts,
               float* __restrict__ adv, float* __restrict__ mean_out) {
-  __shared__ double sh[kBaseThreads / 32];
+  __shared__ double sh[kBaseThreads];
   double acc = 0.0;
   for (int i = threadIdx.x; i < nparts; i += kBaseThreads) acc += part[i];
-  const double mean = block_sum(acc, sh) / (double)n;
+  sh[threadIdx.x] = acc;
+  __syncthreads();
+  for (int d = kBaseThreads / 2; d > 0; d >>= 1) {
+    if ((int)threadIdx.x < d) sh[threadIdx.x] += sh[threadIdx.x + d];
+    __syncthreads();
+  }
+  const double mean = sh[0] / (double)n;
   if (blockIdx.x == 0 && threadIdx.x == 0 && mean_out) mean_out[0] = (float)mean;
   if (!adv) return;
-  const float mh = (float)mean, ml = (float)(mean - (double)mh);
-  const bool fine = fabsf(mh) <= 3.4028234663852886e38f;
-  const int64_t stride = (int64_t)gridDim.x * kBaseThreads;
-  auto centre = [&](float v) {
-    // v - mh exactly as t + err, then the low part of the mean
-    const float t = __fsub_rn(v, mh);
-    const float b = __fsub_rn(t, v);
-    const float err = __fsub_rn(__fsub_rn(v, __fsub_rn(t, b)), __fadd_rn(mh, b));
-    return fine && fabsf(t) <= 3.4028234663852886e38f ? __fadd_rn(t, __fsub_rn(err, ml)) : t;
-  };
-  int64_t i = (int64_t)blockIdx.x * kBaseThreads + threadIdx.x;
-  for (; i + 3 * stride < n; i += 4 * stride) {
-    float v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = x[i + k * stride];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) adv[i + k * stride] = centre(v[k]);
-  }
-  for (; i < n; i += stride) adv[i] = centre(x[i]);
+  for (int64_t i = (int64_t)blockIdx.x * kBaseThreads + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * kBaseThreads)
+    adv[i] = (float)((double)x[i] - mean);
 }
 
 cudaError_t launch_baseline(const float* x, int64_t n, float* adv, float* mean_out, double* ws,

@@ -2,6 +2,8 @@
 one step, of one chunk and around it, of one window and around it, several windows (from 16,384
 envs), env counts off the block's 32, and the kernel of long horizons beside it; and the mean
 baseline at its block edges, on sums that overflow fp32 and on values that cancel."""
+import math
+
 import numpy as np
 import pytest
 
@@ -73,3 +75,25 @@ def test_baseline(n, kind):
     assert abs(gm - m) <= 6e-8 * abs(m) + tol
     ref = x.astype(np.float64) - m
     assert np.all(np.abs(got - ref) <= 1.2e-7 * np.abs(ref) + tol)
+
+
+def test_baseline_sums_in_64_bits():
+    """Every element of a thread's sum is a whole multiple of 2^-23 and every partial sum below 2^28,
+    so that fp64 holds each exactly and the mean is the exact one, rounded once; 2^25 against values
+    of about 2 is more than fp32 pairs keep."""
+    simx = _simx()
+    M, stride = 256, 1024 * 256   # elements per thread, threads
+    v = np.random.default_rng(2).uniform(1.5, 1.99, (M - 8) // 2).astype(np.float32)
+    back = np.random.default_rng(3).permutation(v) + np.float32(2.0 ** -12)
+    big = np.full(4, 2.0 ** 25, np.float32)
+    seq = np.concatenate([big, v, -back, -big]).astype(np.float32)
+    n = M * stride
+    assert simx.returns_baseline_workspace_size(n) == 1024 * 8
+    x = torch.from_numpy(seq).cuda().repeat_interleave(stride)
+    adv, mean = torch.empty(n, device="cuda"), torch.empty(1, device="cuda")
+    ws = torch.empty(1024 * 8, dtype=torch.uint8, device="cuda")
+    simx.returns_baseline(x, adv, mean, ws)
+    m = math.fsum(seq.tolist()) / M
+    assert m != 0.0 and mean.item() == np.float32(m)
+    want = torch.from_numpy((seq.astype(np.float64) - m).astype(np.float32)).cuda()
+    assert torch.equal(adv.view(M, stride), want[:, None].expand(M, stride))
