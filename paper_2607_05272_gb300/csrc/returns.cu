@@ -6,18 +6,19 @@
 // REINFORCE: x = G, delta_t = r_t, c_t = gamma (1 - d_t), x_T = last_value;
 // GAE:       x = A, delta_t = r_t + gamma (1 - d_t) V_{t+1} - V_t,
 //            c_t = gamma lambda (1 - d_t), x_T = 0.
-// Large env counts with 16-byte aligned rows take k_returns_wide: one thread owns four
+// Env counts from 65,536 with 16-byte aligned rows take k_returns_wide: one thread owns four
 // adjacent envs for the whole horizon (one pass: every input read once, every output
 // written once, 17 bytes per sample for GAE), loading 8 time steps ahead with 16-byte
-// loads, so a block reads 1 KB of each row per step.  Otherwise a block owns 32 envs
-// (threadIdx.x) and S chunks of 8 steps at a time (threadIdx.y), held in registers.  Each thread
-// composes its chunk's map x_{t0} = a x_{t1} + b, one thread per env chains the S maps in shared
-// memory, then every thread replays its chunk from the right carry.  Loads are coalesced across
-// envs; no global scratch is needed.  Bound by HBM: 20.5 us at 16,384 envs x 256, inputs not in
-// L2 (k_returns_long 22.5); 234 us at 60,000 x 1024 (300).  Long horizons of few envs would walk
-// many windows, each a round trip to memory and three barriers: they take k_returns_long, whose
-// threads each read a chunk of up to T / 32 steps twice without a barrier between (4003 envs x
-// 1960: 35 us against 44; 64 x 2048: 20 against 29).
+// loads, so a block reads 1 KB of each row per step.
+// Otherwise a block owns 32 envs (threadIdx.x) and S chunks of the horizon (threadIdx.y).  Each
+// thread composes its chunk's map x_{t0} = a x_{t1} + b, one thread per env chains the S maps in
+// shared memory, then every thread replays its chunk from the right carry.  Loads are coalesced
+// across envs; no global scratch is needed.
+//   k_returns_long: chunks of ceil(T / S) steps, read twice, no barrier between a chunk's steps.
+//   k_returns_gae (many envs, see kOnceMinEnvs): windows of S chunks of 8 steps held in registers,
+//   every input read once; each window is a round trip to memory and three barriers.  Past L2
+//   HBM bounds it (60,000 envs x 1024 238 us, 4.4 TB/s, k_returns_long 299); below, the latency of
+//   that round trip (16,384 envs x 256: 18.4 us, 3.9 TB/s, with the buffers not in L2, against 20.4).
 #include <cstdint>
 
 #include "kernels.h"
@@ -130,6 +131,8 @@ k_returns_gae(const float* __restrict__ rew, const float* __restrict__ val,
   }
 }
 
+// A block owns 32 envs and up to 32 chunks of ceil(T / S) steps, each read twice.  Everything below
+// kOnceMinEnvs keeps this composition: training runs carry a last bit of it on.
 __global__ void __launch_bounds__(1024)
 k_returns_long(const float* __restrict__ rew, const float* __restrict__ val,
               const uint8_t* __restrict__ done, const float* __restrict__ last_val, int64_t T,
@@ -205,7 +208,13 @@ k_returns_long(const float* __restrict__ rew, const float* __restrict__ val,
 constexpr int kWideU = 8;                 // time steps loaded ahead
 constexpr int kWideThreads = 64;          // 256 envs per block: every SM gets blocks from 65,536 envs
 constexpr int64_t kWideMinEnvs = 65536;
-constexpr int64_t kOnceMinEnvs = 16384;   // below, windows of k_returns_gae only where one is the horizon
+// The lines of k_returns_gae.  GAE, us with the buffers in L2 and not, k_returns_long against it:
+// 10,000 envs x 256 10.9 and 16.7 against 11.3 and 15.9; 16,383 15.1 and 22.4 against 14.5 and 18.8;
+// 20,000 17.5 and 26.6 against 19.8 and 25.6; 16,384 x 1024 82 against 63.  REINFORCE, a third
+// less to read: 16,384 x 512 16.1 and 23.5 against 23.4 and 26.5, x 1024 44.5 against 50.5; 30,000 x
+// 1024 91.3 against 86.3.
+constexpr int64_t kOnceMinEnvs = 16384;
+constexpr int64_t kOnceMinSamples = 24 << 20;   // REINFORCE
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
@@ -291,27 +300,19 @@ cudaError_t launch_returns_gae(const float* rew, const float* val, const uint8_t
     count_launches(1);
     return cudaGetLastError();
   }
-  // one window covers the horizon, or HBM bounds the walk over several: each input read once
-  if (T <= kRetMaxChunks * kRetL || E >= kOnceMinEnvs) {
+  const bool once = E >= kOnceMinEnvs && (gae || T * E >= kOnceMinSamples);
+  int S = 1;
+  if (once) {
     // Chunks per window: about 130k threads, whose loads in flight cover the memory latency, in
     // one wave of blocks; no more chunks than the horizon has.
-    int S = 1;
     while (S < kRetMaxChunks && E * S * 2 <= 160000 && (int64_t)S * kRetL < T) S *= 2;
-    const dim3 block(32, S);
-    const dim3 grid((unsigned)((E + 31) / 32));
-    if (gae)
-      k_returns_gae<true><<<grid, block, 0, s>>>(rew, val, done, last_val, T, E, ld, gamma, lam, ret, adv);
-    else
-      k_returns_gae<false><<<grid, block, 0, s>>>(rew, val, done, last_val, T, E, ld, gamma, lam, ret, adv);
-    count_launches(1);
-    return cudaGetLastError();
+  } else {
+    // Enough (env, chunk) threads to fill the GPU: ~300k threads, chunks of >= 16 steps.
+    while (S < kRetMaxChunks && E * S * 2 <= 311296 && T / (S * 2) >= 16) S *= 2;
   }
-  // Enough (env, chunk) threads to fill the GPU: ~300k threads, chunks of >= 16 steps.
-  int S = 1;
-  while (S < kRetMaxChunks && E * S * 2 <= 311296 && T / (S * 2) >= 16) S *= 2;
-  const dim3 block(32, S);
-  const dim3 grid((unsigned)((E + 31) / 32));
-  k_returns_long<<<grid, block, 0, s>>>(rew, val, done, last_val, T, E, ld, gamma, lam, ret, adv);
+  const auto kernel = !once ? k_returns_long : gae ? k_returns_gae<true> : k_returns_gae<false>;
+  kernel<<<(unsigned)((E + 31) / 32), dim3(32, S), 0, s>>>(rew, val, done, last_val, T, E, ld, gamma,
+                                                           lam, ret, adv);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -1,7 +1,8 @@
-"""Returns and GAE (Sec. 4.3) by the kernel that reads each input once, at its edges: horizons of
-one step, of one chunk and around it, of one window and around it, several windows (from 16,384
-envs), env counts off the block's 32, and the kernel of long horizons beside it; and the mean
-baseline at its block edges, on sums that overflow fp32 and on values that cancel."""
+"""Returns and GAE (Sec. 4.3) at the edges of the kernel that reads each input once (GAE from 16,384
+envs): horizons of one step, of one chunk and around it, of one window and around it, several
+windows, env counts off the block's 32; returns past its line of 24 Mi samples; and at the same
+horizons the kernel of fewer envs; and the mean baseline at its block edges, on sums that overflow
+fp32 and on values that cancel."""
 import math
 
 import numpy as np
@@ -21,7 +22,8 @@ def _simx():
 
 
 @pytest.mark.parametrize("T,E", [(1, 1), (7, 33), (8, 32), (9, 31), (63, 100), (255, 17), (256, 5),
-                                 (257, 5), (300, 16384), (64, 16391), (129, 40001)])
+                                 (257, 5), (300, 16384), (64, 16391), (129, 40001),
+                                 (1, 16384), (8, 16385), (9, 16390), (65, 16384), (513, 50001)])
 @pytest.mark.parametrize("gae", [False, True], ids=["reinforce", "gae"])
 def test_returns(T, E, gae):
     simx = _simx()
