@@ -162,7 +162,7 @@ __device__ __forceinline__ uint32_t next_chunk(const RolloutArgs& A, const Grp<G
   const U4 w = philox(j, env, kStreamArrival, 0u, A.key0, A.key1);
   const uint32_t gap = TR ? A.tr_gap[j % A.tr_n]
                           : duration_us(__fmul_rn(A.cfg.cand_mean_gap_us, expo1(w.x)));
-  const uint64_t t64 = (uint64_t)s.cT + g.scan_incl(gap);
+  const uint64_t t64 = (uint64_t)s.cT + (TR ? g.scan_clamp(gap) : g.scan_incl(gap));
   c.over = t64 >= kTimeLimit;
   c.T = c.over ? kTimeLimit : (uint32_t)t64;
   c.wy = w.y;

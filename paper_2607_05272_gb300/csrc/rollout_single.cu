@@ -127,7 +127,7 @@ __device__ __forceinline__ void refill(const RolloutArgs& A, const Window& win, 
   for (int q = 0; q < Q; ++q) r[q] = philox(fj + 32u * q + lane, env, kStreamArrival, 0u, A.key0, A.key1);
 #pragma unroll
   for (int q = 0; q < Q; ++q)
-    sum[q] = TR ? A.tr_gap[(fj + 32u * q + lane) % A.tr_n]
+    sum[q] = TR ? min(A.tr_gap[(fj + 32u * q + lane) % A.tr_n], kTimeLimit)
                 : duration_us(__fmul_rn(c.cand_mean_gap_us, expo1(r[q].x)));
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -136,7 +136,10 @@ __device__ __forceinline__ void refill(const RolloutArgs& A, const Window& win, 
     for (int q = 0; q < Q; ++q) y[q] = __shfl_up_sync(0xFFFFFFFFu, sum[q], d);
 #pragma unroll
     for (int q = 0; q < Q; ++q)
-      if (lane >= (uint32_t)d) sum[q] += y[q];
+      if (lane >= (uint32_t)d) {
+        sum[q] += y[q];
+        if (TR) sum[q] = min(sum[q], kTimeLimit);   // a trace's gaps may add up past 32 bits
+      }
   }
 #pragma unroll
   for (int q = 0; q < Q; ++q) {

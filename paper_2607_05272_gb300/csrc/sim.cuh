@@ -144,6 +144,17 @@ struct Grp {
     }
     return v;
   }
+  // The same of durations, clamped at the time limit (as the time that they add up to is): a
+  // replayed trace's gaps may add up past 32 bits within one group, drawn ones (2^26 each) do not.
+  __device__ __forceinline__ uint32_t scan_clamp(uint32_t v) const {
+    v = v < kTimeLimit ? v : kTimeLimit;
+#pragma unroll
+    for (int d = 1; d < G; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(mask, v, d, G);
+      if (gl >= (uint32_t)d) v = v + y < kTimeLimit ? v + y : kTimeLimit;
+    }
+    return v;
+  }
   __device__ __forceinline__ void sync() const { __syncwarp(mask); }
 };
 

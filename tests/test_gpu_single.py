@@ -85,3 +85,40 @@ def test_single_rollout(cfg, hidden, acts, mode, H, new, request, monkeypatch):
     assert np.array_equal(col["trace"], ref["trace"])
     for k in ("obs", "reward", "logp", "value"):
         assert np.array_equal(col[k].view(np.uint32), ref[k].view(np.uint32)), k
+
+
+@pytest.mark.parametrize("gap,H", [((1 << 27) + 7, 12), (1 << 28, 5)])
+@pytest.mark.parametrize("name,E", [("c2t", 2500), ("c2t", 40), ("c3t", 300)])
+@pytest.mark.parametrize("stage", ["", "0"], ids=["default", "lanes"])
+def test_long_gaps(name, E, gap, H, stage, monkeypatch):
+    """A trace whose gaps add up past 32 bits within one group of candidates: their times end at the
+    limit, which no decision here reaches, and none starts over."""
+    from paper_2607_05272_gb300 import build as B
+    B.build()
+    from paper_2607_05272_gb300 import simx
+    for k in ("SIMX_LANES", "SIMX_THREADS"):
+        monkeypatch.delenv(k, raising=False)
+    monkeypatch.setenv("SIMX_STAGE", stage)
+    cfg = W.CONFIGS[name](E)
+    cfg["trace"] = (np.full(64, gap, np.uint32), None, None)
+    dims, hv = W.mlp_dims(name)
+    Ws, bs = W.policy_weights(name, dims, 7)
+    acts = W.mlp_acts(name)
+    pol = simx.Policy([torch.from_numpy(w).cuda() for w in Ws], [torch.from_numpy(b).cuda() for b in bs],
+                      hv, acts)
+    sim = simx.Sim(cfg)
+    sim.reset(0xB23)
+    buf = simx.alloc_rollout(E, sim.D, H, has_value=hv, trace=True)
+    sim.rollout("sample", H, buf, pol)
+    torch.cuda.synchronize()
+    envs = sorted({0, 7, E // 2, E - 1})
+    sel = torch.tensor(envs, device="cuda")
+    ref = oracle.rollout(cfg, (Ws, bs, hv, acts), 0xB23, 0, envs, H)
+    col = {k: v.index_select(v.dim() - 1, sel).cpu().numpy() for k, v in buf.items()}
+    assert np.array_equal(col["action"], ref["action"].astype(np.uint8))
+    assert np.array_equal(col["trace"], ref["trace"])
+    for k in ("obs", "reward", "logp"):
+        assert np.array_equal(col[k].view(np.uint32), ref[k].view(np.uint32)), k
+    assert np.array_equal(sim.save()[envs], ref["state"])
+    assert sim.last_status() == (0, 0)
+    sim.close()
