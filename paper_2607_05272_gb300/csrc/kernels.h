@@ -86,6 +86,15 @@ struct PolicyArgs {
 // spreads them over all 32.
 int act_stride_pad(const DevMlp& m, int B, int threads);
 
+// Lets a kernel be launched with up to `most` bytes of dynamic shared memory: the most that any of
+// its plans takes, the same on every call, so that host threads that launch the kernel with plans of
+// different sizes never lower the limit between another's setting and its launch.
+template <class K>
+inline cudaError_t allow_smem(K* kernel, int most) {
+  return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+constexpr int kMaxSmem = 227 * 1024;   // per block, the kernel's static shared memory included
+
 cudaError_t launch_rollout(const RolloutArgs& a, cudaStream_t s);
 // rollout_route.cu: the router's rollout with one simulator thread per env
 size_t plan_route(RolloutArgs& a);

@@ -31,6 +31,7 @@ namespace {
 constexpr int NT = 512;          // threads
 constexpr int kMaxRows = 64;     // rows per tile at most
 constexpr int kLanes = NT / kMaxRows;   // lanes per row in the gather and the loss head
+constexpr int kMostSmem = kMaxSmem - 2048;   // the static statistics and a margin
 
 struct BlockLoss {
   LossArgs a;
@@ -406,7 +407,7 @@ BlockPlan plan(const LossArgs& a) {
   for (p.R = 8; p.R <= kMaxRows && (a.n + p.R - 1) / p.R > sms;) p.R += 8;
   if (p.R > kMaxRows) return p;
   p.smem = ((size_t)rows * (p.R + 4) + wfl + nb) * sizeof(float) + 16;
-  if (p.smem > 225 * 1024) return p;   // 227 KB less a margin for the static statistics
+  if (p.smem > (size_t)kMostSmem) return p;
   p.grid = (int)((a.n + p.R - 1) / p.R);
   int off = rows * (p.R + 4);
   for (int l = 0; l < L; ++l) {
@@ -478,7 +479,7 @@ cudaError_t launch_loss_block(const LossArgs& a, void* ws, size_t ws_bytes, cuda
   F.part = reinterpret_cast<float*>(base + p.part_off);
   F.spart = reinterpret_cast<double*>(base + p.spart_off);
   launch_pack_loss_w(pk, s);
-  cudaFuncSetAttribute(k_loss_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+  if (const cudaError_t e = allow_smem(k_loss_block, kMostSmem)) return e;
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)p.grid);
   lc.blockDim = dim3((unsigned)NT);

@@ -725,7 +725,7 @@ cudaError_t launch_loss_fused(const LossArgs& a, void* ws, size_t ws_bytes, cuda
   }
   auto k = p.R == 64 ? (p.resident ? k_loss_fused<64, 2> : k_loss_fused<64, 0>)
                      : (p.stage ? k_loss_fused<32, 1> : k_loss_fused<32, 0>);
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+  if (const cudaError_t e = allow_smem(k, kMaxSmem - 2 * 1024)) return e;   // the static statistics
   k<<<p.grid, kLThreads, p.smem, s>>>(F);
   launch_loss_reduce(F.part, p.grid, p.n_params, F.spart, a, s);
   count_launches(1);

@@ -716,7 +716,7 @@ cudaError_t launch_loss_tc(const LossArgs& a, void* ws, size_t ws_bytes, cudaStr
   A.part = reinterpret_cast<float*>(base + w.part);
   A.spart = reinterpret_cast<double*>(base + w.spart);
   A.ntiles = (a.n + tcl::kR - 1) / tcl::kR;
-  cudaFuncSetAttribute(tcl::k_loss_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+  if (const cudaError_t e = allow_smem(tcl::k_loss_tc, kMaxSmem - 4 * tcl::kR * 8)) return e;
   tcl::k_loss_tc<<<w.grid, tcl::kThreads, p.smem, s>>>(A);
   launch_loss_reduce(A.part, w.grid, p.n_params, A.spart, a, s);
   count_launches(1);

@@ -1074,7 +1074,7 @@ cudaError_t launch_loss_wide(const LossArgs& a, void* ws, size_t ws_bytes, cudaS
   if (blocks > cap) blocks = cap;
   lw::k_lw_prep<<<(unsigned)blocks, 256, 0, s>>>(A);
   // a cluster of two CTAs per 128-row tile
-  cudaFuncSetAttribute(lw::k_lw_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+  if (const cudaError_t e = allow_smem(lw::k_lw_rows, kMaxSmem)) return e;
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)(2 * p.ntiles));
   lc.blockDim = dim3(lw::kThreads);
@@ -1093,7 +1093,7 @@ cudaError_t launch_loss_wide(const LossArgs& a, void* ws, size_t ws_bytes, cudaS
   lc.numAttrs = 2;
   cudaError_t e = cudaLaunchKernelEx(&lc, lw::k_lw_rows, A);
   if (e != cudaSuccess) return e;
-  cudaFuncSetAttribute(lw::k_lw_dw, cudaFuncAttributeMaxDynamicSharedMemorySize, p.dw_smem);
+  if ((e = allow_smem(lw::k_lw_dw, kMaxSmem)) != cudaSuccess) return e;
   lc.gridDim = dim3((unsigned)(p.mt_total * p.S));
   lc.blockDim = dim3(lw::kDwThreads);
   lc.dynamicSmemBytes = (size_t)p.dw_smem;

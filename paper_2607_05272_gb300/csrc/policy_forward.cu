@@ -178,7 +178,7 @@ cudaError_t launch_policy_block(const PolicyArgs& p, cudaStream_t s) {
   auto k = p.mlp.grid ? (p.fwd.big ? k_forward_block<2, true, true> : k_forward_block<3, false, true>)
                       : (p.fwd.big ? k_forward_block<2, true, false> : k_forward_block<3, false, false>);
   const size_t sh = fwd_smem(p.fwd);
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+  if (const cudaError_t e = allow_smem(k, kMaxSmem)) return e;
   k<<<(unsigned)p.fwd.sms, 256, sh, s>>>(p);
   count_launches(1);
   return cudaGetLastError();

@@ -1400,7 +1400,7 @@ static size_t plan_stage_forward(RolloutArgs& a, int B, const void* kfn) {
   P.S = 2;
   if (!stage_tiles(m, B, a.threads, P)) return plain;
   int r0 = 0;
-  cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (allow_smem(kfn, kMaxSmem) != cudaSuccess) return plain;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r0, kfn, a.threads, plain) != cudaSuccess) {
     cudaGetLastError();
     return plain;
@@ -1479,7 +1479,7 @@ static cudaError_t rollout_t(const RolloutArgs& a0, cudaStream_t s) {
   RolloutArgs a = a0;
   const size_t sh = plan_rollout_t<ROUTE, G>(a);
   auto k = pick_rollout<ROUTE, G>(a);
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+  if (const cudaError_t e = allow_smem(k, kMaxSmem)) return e;
   k<<<grid_for(a.st.E, a.threads / G), a.threads, sh, s>>>(a);
   count_launches(1);
   return cudaGetLastError();
@@ -1497,7 +1497,7 @@ template <bool ROUTE, int G>
 static cudaError_t observe_t(const RolloutArgs& a, cudaStream_t s) {
   const int B = a.threads / G;
   const size_t sh = env_smem(a, B);
-  cudaFuncSetAttribute(k_observe<ROUTE, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+  if (const cudaError_t e = allow_smem(k_observe<ROUTE, G>, kMaxSmem)) return e;
   k_observe<ROUTE, G><<<grid_for(a.st.E, B), a.threads, sh, s>>>(a);
   count_launches(1);
   return cudaGetLastError();
@@ -1558,7 +1558,7 @@ template <int G>
 static cudaError_t policy_forward_t(const PolicyArgs& p, cudaStream_t s) {
   const int B = p.threads / G;
   const size_t sh = ((size_t)2 * p.maxd4 * (B + 4) + (size_t)p.apad * B) * sizeof(float);
-  cudaFuncSetAttribute(k_policy_forward<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+  if (const cudaError_t e = allow_smem(k_policy_forward<G>, kMaxSmem)) return e;
   k_policy_forward<G><<<grid_for(p.n, B), p.threads, sh, s>>>(p);
   count_launches(1);
   return cudaGetLastError();

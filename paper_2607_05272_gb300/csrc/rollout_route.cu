@@ -522,7 +522,7 @@ size_t plan_route(RolloutArgs& a) {
 
 cudaError_t launch_route(const RolloutArgs& a, size_t sh, cudaStream_t s) {
   const void* k = pick_kernel(a);
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+  if (const cudaError_t e = allow_smem(k, kMaxSmem)) return e;
   const int NE = a.threads / a.G;
   void* args[] = {const_cast<RolloutArgs*>(&a)};
   const cudaError_t e = cudaLaunchKernel(k, dim3((a.st.E + NE - 1) / NE), dim3(a.threads), args, sh, s);

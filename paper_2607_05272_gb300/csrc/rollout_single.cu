@@ -648,7 +648,7 @@ cudaError_t launch_single(const RolloutArgs& a, size_t sh, cudaStream_t s) {
   const bool tr = a.cfg.arrival_kind == SIMX_ARR_TRACE;
   auto k = a.mlp.grid ? (tr ? k_single<true, true> : k_single<false, true>)
                       : (tr ? k_single<true, false> : k_single<false, false>);
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+  if (const cudaError_t e = allow_smem(k, kMaxSmem)) return e;
   const int NE = a.threads / a.G;
   k<<<(a.st.E + NE - 1) / NE, a.threads, sh, s>>>(a);
   count_launches(1);

@@ -60,3 +60,53 @@ def test_policy_forward(n, dims, acts, mode):
                                      {"sample": 0, "argmax": 1}[mode], 77, 9, 40 + i)
         assert np.array_equal(got["logits"][:, i].view(np.uint32), lg.view(np.uint32))
         assert got["value"][i] == v and got["action"][i] == a and got["logp"][i] == lp
+
+
+def test_host_threads_with_plans_of_different_sizes():
+    """policy_forward_ws shares no state between calls: two host threads whose launches of one kernel
+    ask for different amounts of shared memory, on streams and workspaces of their own."""
+    import threading
+    from paper_2607_05272_gb300 import build as B
+    B.build()
+    from paper_2607_05272_gb300 import simx
+    rng = np.random.default_rng(5)
+
+    def make(dims, n):
+        Ws = [torch.from_numpy((0.3 * rng.standard_normal((b, a))).astype(np.float32)).cuda()
+              for a, b in zip(dims[:-1], dims[1:])]
+        pol = simx.Policy(Ws, [torch.zeros(b, device="cuda") for b in dims[1:]], True)
+        return dict(pol=pol, obs=torch.randn((dims[0], n), device="cuda"), n=n,
+                    ws=torch.empty(simx.policy_forward_workspace_size(pol), dtype=torch.uint8, device="cuda"),
+                    logits=torch.empty((dims[-1] - 1, n), device="cuda"), stream=torch.cuda.Stream())
+
+    def call(s):
+        simx.policy_forward(s["pol"], s["obs"], s["n"], "sample", 1, 2, logits=s["logits"],
+                            workspace=s["ws"], stream=s["stream"].cuda_stream)
+
+    # both take the kernel with 8 x 8 tiles, one with small and one with large activations and stages
+    jobs = [make([8, 132, 5], 12000), make([28, 256, 256, 49], 12000)]
+    want, errors = [], []
+    for s in jobs:
+        call(s)
+        torch.cuda.synchronize()
+        want.append(s["logits"].clone())
+    start = threading.Barrier(2)
+
+    def work(s):
+        try:
+            start.wait()
+            for _ in range(1500):
+                call(s)
+        except Exception as e:   # noqa: BLE001 (reported below)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(s,)) for s in jobs]
+    torch.cuda.synchronize()
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    for s, w in zip(jobs, want):
+        assert torch.equal(s["logits"], w)
