@@ -336,7 +336,8 @@ simx_status simx_launch_shape(simx_ctx* ctx, const simx_mlp* pol, int policy_mod
  * The policy is repacked into a buffer the library keeps per device: calls on one device
  * must not overlap on the GPU, and a call with a larger policy replaces the buffer (a
  * CUDA graph that captured an earlier call would then use freed memory).  For concurrent
- * streams or graph capture use policy_forward_ws.
+ * streams or graph capture use policy_forward_ws.  If a bounded wait for a staged copy of
+ * the weights runs out, the float outputs of the columns concerned are NaN.
  */
 simx_status policy_forward(const simx_mlp* pol, const float* d_obs, int64_t ld, int64_t n,
                            int policy_mode, uint64_t seed, uint32_t step, uint32_t env_base,

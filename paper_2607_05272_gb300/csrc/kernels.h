@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <cstdlib>
 
 #include "../../include/simx.h"
 #include "sim.cuh"
@@ -92,6 +93,12 @@ int act_stride_pad(const DevMlp& m, int B, int threads);
 template <class K>
 inline cudaError_t allow_smem(K* kernel, int most) {
   return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+// Weight copies withheld at the end of each block's sequence (SIMX_WITHHOLD_COPIES, 0 without it): a
+// wait that nothing ends, for the tests of what a call reports when a bounded wait runs out.
+inline uint32_t copies_withheld() {
+  const char* v = getenv("SIMX_WITHHOLD_COPIES");
+  return v ? (uint32_t)atoi(v) : 0u;
 }
 constexpr int kMaxSmem = 227 * 1024;   // per block, the kernel's static shared memory included
 

@@ -35,6 +35,10 @@ __global__ void __launch_bounds__(256, MINB) k_forward_block(const __grid_consta
     const bool live = col < A.n;
     for (int d = part; d < D; d += G) smem[d * ld + slot] = live ? __ldg(A.obs + (int64_t)d * A.ld + col) : 0.0f;
     fwd::forward<BIG, GRID, false>(m, P, p, at, smem, NE, ld, vt, []() {});
+    if (*p.flag) {   // a wait for weights ran out: every output from here on says so
+      for (int j = part; j < m.dims[m.n_layers]; j += G) smem[j * ld + slot] = __uint_as_float(0x7FC00000u);
+      __syncthreads();
+    }
     const float* z = smem + slot;
     if (live && A.logits)
       for (int j = part; j < NA; j += G) A.logits[(int64_t)j * A.ld + col] = z[j * ld];
@@ -169,6 +173,7 @@ bool plan_policy_block(PolicyArgs& p) {
   if (!fwd_plan_stages(m, off, (size_t)(227 * 1024) / (size_t)per_sm - 1024, P)) return false;
   P.side_layer = -1;
   P.sms = (int)(per_sm * sms < tiles ? per_sm * sms : tiles);   // the grid
+  P.withheld = copies_withheld();
   P.on = 1;
   p.fwd = P;
   return true;

@@ -513,6 +513,7 @@ size_t plan_route(RolloutArgs& a) {
       P.side_vt = nact;
     }
   }
+  P.withheld = copies_withheld();
   P.on = 1;
   a.fwd = P;
   a.G = G;

@@ -637,6 +637,7 @@ size_t plan_single(RolloutArgs& a) {
   if (!fwd_plan_resident(m, off, half, P) && !fwd_plan_stages(m, off, half, P)) return 0;
   P.side_layer = -1;
   P.sms = (int)sms;
+  P.withheld = copies_withheld();
   P.on = 1;
   a.fwd = P;
   a.G = G;

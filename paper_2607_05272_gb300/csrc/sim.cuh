@@ -93,6 +93,7 @@ struct FwdPlan {
   // = the layers), layer l's at byte woff[l] after `off`
   int resident;
   uint32_t woff[SIMX_MAX_LAYERS];
+  uint32_t withheld;           // chunks at the end of the launch's sequence never issued (tests)
   // rollout_single.cu: byte offsets of the envs' chunks of candidates and of the requests' rings
   // (0: those stay in global memory)
   uint32_t win_off, ring_off;
