@@ -44,6 +44,7 @@ struct BlockLoss {
   int poff[SIMX_MAX_LAYERS];
   int n_params, R, ld;
   int bar_off;                       // bytes
+  int withheld;                      // the last copy is never issued (tests)
   float* part;
   double* spart;
 };
@@ -195,7 +196,8 @@ __global__ void __launch_bounds__(NT, 1) k_loss_block(const __grid_constant__ Bl
       total += (uint32_t)(a.dims[l] * F.npad[l] + (l ? a.dims[l + 1] * F.kpad[l] : 0)) * 4u;
     tcx::mbar_arrive_expect_tx(bar, total);
     for (int l = 0; l < L; ++l) {
-      tcx::bulk_g2s(sm + F.wt_off[l], F.Wt[l], (uint32_t)(a.dims[l] * F.npad[l]) * 4u, bar);
+      if (l + 1 < L || !F.withheld)
+        tcx::bulk_g2s(sm + F.wt_off[l], F.Wt[l], (uint32_t)(a.dims[l] * F.npad[l]) * 4u, bar);
       if (l) tcx::bulk_g2s(sm + F.wn_off[l], F.Wn[l], (uint32_t)(a.dims[l + 1] * F.kpad[l]) * 4u, bar);
     }
   }
@@ -360,12 +362,13 @@ __global__ void __launch_bounds__(NT, 1) k_loss_block(const __grid_constant__ Bl
     sstat[tid / 32][2] = st_h;
     sstat[tid / 32][3] = st_cf;
   }
-  __syncthreads();
+  const bool bad = __syncthreads_or(!fine);
+  if (bad)   // the weights never landed: the gradient and the statistics say so
+    for (int i = tid; i < F.n_params; i += NT) part[i] = __uint_as_float(0x7FC00000u);
   if (tid < 4) {
     double v = 0.0;
     for (int w = 0; w < NT / 32; ++w) v += sstat[w][tid];
-    // the weights never landed: say so in the statistics
-    F.spart[(size_t)blockIdx.x * 4 + tid] = fine ? v : __longlong_as_double(0x7FF8000000000000LL);
+    F.spart[(size_t)blockIdx.x * 4 + tid] = bad ? __longlong_as_double(0x7FF8000000000000LL) : v;
   }
 }
 
@@ -476,6 +479,7 @@ cudaError_t launch_loss_block(const LossArgs& a, void* ws, size_t ws_bytes, cuda
   F.R = p.R;
   F.ld = p.R + 4;
   F.bar_off = p.bar_off;
+  F.withheld = copies_withheld() != 0u;
   F.part = reinterpret_cast<float*>(base + p.part_off);
   F.spart = reinterpret_cast<double*>(base + p.spart_off);
   launch_pack_loss_w(pk, s);

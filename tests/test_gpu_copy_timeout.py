@@ -68,3 +68,31 @@ def test_rollout_flags_its_envs(name, E, hidden, monkeypatch):
     assert st != 0 and code == 16   # SIMX_DEV_COPY_TIMEOUT
     assert int(buf["action"].max()) < pol.n_actions
     sim.close()
+
+
+def test_loss_gradient_says_nan(monkeypatch):
+    """The FP32 loss of one tile per SM: gradient and statistics, so that no optimiser step takes a
+    gradient of unloaded weights for a finite one."""
+    simx = _simx()
+    pol = _policy(simx, "c3")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 32 * sms + 1   # the first size of the block kernel
+    g = torch.Generator("cuda").manual_seed(2)
+    buf = dict(obs=torch.randn((1, 13, n), device="cuda", generator=g),
+               action=torch.randint(0, 16, (1, n), device="cuda", generator=g, dtype=torch.uint8),
+               logp=torch.full((1, n), -2.7, device="cuda"))
+    adv, ret = torch.randn((2, 1, n), device="cuda", generator=g)
+    ws = torch.empty(simx.ppo_loss_grad_workspace_size(pol, n), dtype=torch.uint8, device="cuda")
+
+    def call():
+        grad, stats = torch.zeros(pol.n_params, device="cuda"), torch.zeros(5, device="cuda")
+        simx.ppo_loss_grad(pol, buf, ret, adv, None, n, "ppo", 0.2, 0.5, 0.01, grad, stats, ws)
+        torch.cuda.synchronize()
+        return grad, stats
+
+    good = call()
+    monkeypatch.setenv("SIMX_WITHHOLD_COPIES", "1")
+    grad, stats = call()
+    monkeypatch.delenv("SIMX_WITHHOLD_COPIES")
+    assert bool(torch.isnan(grad).all()) and bool(torch.isnan(stats[:4]).all())
+    assert all(torch.equal(a, b) for a, b in zip(good, call())) and bool(torch.isfinite(good[0]).all())
