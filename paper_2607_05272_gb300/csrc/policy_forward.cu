@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(256, MINB) k_forward_block(const __grid_consta
     }
     __syncthreads();   // the next tile's observations replace the logits
   }
-  if (vt == producer && *p.flag) fwd::drain(P, p, at);
+  if (vt == producer && *p.flag) fwd::drain(P, p);
 }
 
 bool fwd_pick_tiles(const DevMlp& m, int NE, int threads, bool big, int pct, FwdPlan& P) {

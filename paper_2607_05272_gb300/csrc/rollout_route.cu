@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(NT, MINB) k_route(const __grid_constant__ Roll
     phase_step<TR>(A, smem, t);
   }
   __syncthreads();
-  if (vt == producer && *p.flag) fwd::drain(P, p, at);
+  if (vt == producer && *p.flag) fwd::drain(P, p);
   {
     const DevState& st = A.st;
     const uint32_t* words = reinterpret_cast<const uint32_t*>(sb + P.st_off);

@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(256, 3) k_single(const __grid_constant__ Rollo
     const Who w(A, smem);
     observe(A, w, nullptr, 0, A.next_obs + w.env, A.next_ld);
   }
-  if (vt == producer && *p.flag) fwd::drain(P, p, at);
+  if (vt == producer && *p.flag) fwd::drain(P, p);
   for (int i = (int)threadIdx.x; i < W_WORDS * NE; i += (int)blockDim.x) {
     const int w = i >> P.ne_shift, e = i & (NE - 1);
     if (!word_saved(w) || env0 + (uint32_t)e >= st.E) continue;

@@ -13,6 +13,7 @@
 
 #include "../../include/simx.h"
 #include "devmath.cuh"
+#include "pipe_phase.h"
 #include "tc_common.cuh"
 
 namespace simx {
@@ -61,7 +62,7 @@ struct StagePlan {
   int n;                       // chunks per forward
   uint32_t cb;                 // bytes per stage
   uint32_t off;                // first stage
-  uint32_t bar_off;            // S mbarriers (8 B each), then the timeout flag (4 B)
+  uint32_t bar_off;            // S mbarriers (8 B each), then the timeout flag and the chunks issued (4 B each)
   int rpc[SIMX_MAX_LAYERS];    // weight rows per chunk
   int cnt[SIMX_MAX_LAYERS];    // chunks of each layer
   int te[SIMX_MAX_LAYERS], to[SIMX_MAX_LAYERS];   // register tile: envs x outputs
@@ -390,7 +391,7 @@ __device__ __forceinline__ float* mlp_forward_warp(const DevMlp& m, float* X0, f
 struct StagePipe {
   float* stages;
   uint64_t* full;
-  volatile int* flag;
+  volatile int* flag;   // [0] a wait timed out, [1] chunks issued
   uint32_t cc;      // chunks consumed so far in the launch
   uint32_t total;   // chunks the launch consumes (steps x chunks per forward)
 };
@@ -410,6 +411,7 @@ __device__ __forceinline__ void stage_issue(const DevMlp& m, const StagePlan& P,
   const int rows = m.dims[l] - row0 < P.rpc[l] ? m.dims[l] - row0 : P.rpc[l];
   const uint32_t bytes = (uint32_t)(rows * Np) * 4u;
   const uint32_t st = g % (uint32_t)P.S;
+  p.flag[1] = (int)(g + 1u);
   tcx::mbar_arrive_expect_tx(&p.full[st], bytes);
   tcx::bulk_g2s(p.stages + (size_t)st * (P.cb / 4u), m.Wt[l] + (size_t)row0 * Np, bytes,
                 &p.full[st]);
@@ -418,16 +420,18 @@ __device__ __forceinline__ void stage_issue(const DevMlp& m, const StagePlan& P,
 // Thread 0 at launch start: the barriers, then the first S chunks.
 __device__ __forceinline__ void stage_start(const DevMlp& m, const StagePlan& P, const StagePipe& p) {
   for (int i = 0; i < P.S; ++i) tcx::mbar_init(&p.full[i], 1);
-  *p.flag = 0;
+  p.flag[0] = p.flag[1] = 0;
   tcx::mbar_fence_init();
   for (int i = 0; i < P.S; ++i) stage_issue(m, P, p, (uint32_t)i);
 }
 
-// Thread 0 at launch end, after a timeout only: a bounded wait for every stage's copy
-// still in flight, so that none lands after the block has exited.
+// Thread 0 at launch end, after a timeout only: a bounded wait for every stage's last copy
+// issued, so that none lands after the block has exited.
 __device__ __forceinline__ void stage_drain(const StagePlan& P, const StagePipe& p) {
-  for (uint32_t g = p.cc; g < p.cc + (uint32_t)P.S && g < p.total; ++g)
-    tcx::mbar_wait(&p.full[g % (uint32_t)P.S], (g / (uint32_t)P.S) & 1u, 200000000ll);
+  for (int i = 0; i < P.S; ++i) {
+    const int parity = last_parity((uint32_t)p.flag[1], (uint32_t)P.S, (uint32_t)i);
+    if (parity >= 0) tcx::mbar_wait(&p.full[i], (uint32_t)parity, 200000000ll);
+  }
 }
 
 // One layer of the staged forward; returns the chunks consumed so far.
