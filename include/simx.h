@@ -477,6 +477,13 @@ uint64_t simx_launches(void);
 simx_status simx_fma_probe(int64_t iters, float* d_sink, double* host_flops, void* stream);
 size_t simx_fma_probe_sink_floats(void);
 
+/* Check of the elementary functions (no counterpart in the paper): the branch-free forms that the
+   block-wide policy forwards and the FP32 loss evaluate, against the forms that define the bits,
+   over every fp32 input (which = 0: tanh) or every one that is not above zero (which = 1: exp).
+   d_count (device) receives the number of inputs whose results differ in a bit.  SIMX_EINVAL for
+   another `which` or a NULL pointer. */
+simx_status simx_math_check(int which, uint64_t* d_count, void* stream);
+
 const char* simx_strerror(simx_status s);
 const char* simx_last_error(void);
 

@@ -278,6 +278,13 @@ simx_status simx_fma_probe(int64_t iters, float* d_sink, double* host_flops, voi
 
 size_t simx_fma_probe_sink_floats(void) { return fma_probe_sink_floats(); }
 
+simx_status simx_math_check(int which, uint64_t* d_count, void* stream) {
+  if (which < 0 || which > 1 || !d_count) return fail(SIMX_EINVAL, "math check %d", which);
+  const cudaError_t e = launch_math_check(which, reinterpret_cast<unsigned long long*>(d_count), (cudaStream_t)stream);
+  if (e != cudaSuccess) return cuda_fail(e, "math check");
+  return SIMX_OK;
+}
+
 size_t simx_adam_workspace_size(int64_t n) { return n < 1 ? 0 : adam_workspace_bytes(n); }
 
 simx_status simx_adam_step(float* d_params, const float* d_grad, float* d_m, float* d_v,

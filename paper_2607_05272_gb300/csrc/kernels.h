@@ -207,6 +207,8 @@ void launch_loss_reduce(const float* part, int nb, int n_params, const double* s
 // the same with nbs statistics partials (nb gradient partials summed in order)
 void launch_loss_reduce_n(const float* part, int nb, int n_params, const double* spart, int nbs,
                           const LossArgs& a, cudaStream_t s);
+// math_check.cu
+cudaError_t launch_math_check(int which, unsigned long long* count, cudaStream_t s);
 // fma_probe.cu
 cudaError_t launch_fma_probe(int64_t iters, float* sink, double* flops, cudaStream_t s);
 

@@ -114,6 +114,7 @@ SIGNATURES = [
     ("simx_launches", U64, []),
     ("simx_fma_probe", C.c_int, [I64, P, P, P]),
     ("simx_fma_probe_sink_floats", SZ, []),
+    ("simx_math_check", C.c_int, [C.c_int, P, P]),
     ("simx_strerror", C.c_char_p, [C.c_int]),
     ("simx_last_error", C.c_char_p, []),
 ]
@@ -454,3 +455,9 @@ def fma_probe(iters: int, sink, stream=None) -> float:
     fl = C.c_double(0.0)
     _check(lib().simx_fma_probe(iters, _ptr(sink), C.byref(fl), _stream(stream)))
     return fl.value
+
+
+def math_check(which: str, count, stream=None):
+    """Count into `count` (int64 device tensor of one element) the fp32 inputs on which the
+    branch-free "tanh" or "exp" differs from the defining one."""
+    _check(lib().simx_math_check({"tanh": 0, "exp": 1}[which], _ptr(count), _stream(stream)))
