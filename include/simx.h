@@ -328,6 +328,26 @@ simx_status simx_launch_shape(simx_ctx* ctx, const simx_mlp* pol, int policy_mod
                               int32_t* host_out);
 
 /*
+ * Which kernel that launch is, where simx_launch_shape says "fused" of several (host only, for
+ * the same purpose, with the same errors).  host_out[2] receives: [0] 0 = a lane group per env,
+ * 1 = the thread-per-env step of the policy-free modes, 2 = the router's block rollout, 3 = the
+ * single server's; [1] where the policy forward reads its weights: 0 = through L1, 1 = stages of
+ * the lane-group kernel, 2 = the block forward's stages, 3 = resident in shared memory, 4 = the
+ * tensor cores' operand images.
+ */
+simx_status simx_rollout_kernel(simx_ctx* ctx, const simx_mlp* pol, int policy_mode,
+                                int32_t* host_out);
+
+/* The same of policy_forward with n columns: columns per block of the block forward, 0 for the
+   lane-group kernel, -1 for n < 1 or a policy that it would refuse. */
+int32_t simx_forward_columns(const simx_mlp* pol, int64_t n);
+
+/* The same of ppo_loss_grad with n rows: 0 = the GEMM pipeline, 1 = the fused FP32 kernel, 2 = the
+   FP32 kernel of one tile per SM, 3 = the one-SM tensor-core kernel, 4 = the streamed tensor-core
+   kernels, -1 for n < 1 or a policy that it would refuse. */
+int32_t simx_loss_kernel(const simx_mlp* pol, int64_t n, int precision);
+
+/*
  * Batched policy forward (Sec. 4.2) for n observation columns d_obs [dims[0]][ld].
  * Column i is env (env_base + i) at global decision step `step`, which fixes its
  * POLICY Philox counter, so this reproduces the actions the rollout drew.

@@ -553,9 +553,10 @@ simx_status rollout_collect(simx_ctx* c, const simx_mlp* pol, int policy_mode, i
   return SIMX_OK;
 }
 
-simx_status simx_launch_shape(simx_ctx* c, const simx_mlp* pol, int policy_mode,
-                              int32_t* host_out) {
-  if (!c || !host_out) return fail(SIMX_EINVAL, "ctx or host_out is NULL");
+// The launch that rollout_collect makes for this policy and mode: a with its plans, whether it is
+// the thread-per-env step (no repack needed).
+static simx_status rollout_plan(simx_ctx* c, const simx_mlp* pol, int policy_mode, RolloutArgs& a,
+                                bool& thread) {
   const bool route = c->cfg.mode == SIMX_MODE_ROUTE;
   const bool net = policy_mode == SIMX_POLICY_SAMPLE || policy_mode == SIMX_POLICY_ARGMAX;
   if (policy_mode < 0 || policy_mode > SIMX_POLICY_EXTERNAL) return fail(SIMX_EINVAL, "policy_mode %d", policy_mode);
@@ -564,34 +565,48 @@ simx_status simx_launch_shape(simx_ctx* c, const simx_mlp* pol, int policy_mode,
     if (v != SIMX_OK) return v;
   }
   cudaSetDevice(c->device);
-  RolloutArgs a;
   base_args(c, a);
   a.policy_mode = policy_mode;
-  const bool thread = step_thread_supported(a);
+  thread = step_thread_supported(a);
+  if (thread || !net) return SIMX_OK;
+  a.mlp_warp = mlp_warp_of(route, a.G, pol);
+  a.mlp.n_layers = pol->n_layers;
+  for (int l = 0; l <= pol->n_layers; ++l) {
+    a.mlp.dims[l] = pol->dims[l];
+    a.mlp.npad[l] = l ? round_up(pol->dims[l], 4) : pol->dims[0];
+  }
+  a.mlp.grid = pol->grid;
+  act_layout(mlp_maxdim(pol), (int)a.n_actions, a.maxd4, a.apad);
+  a.bs_pad = a.mlp_warp ? act_stride_pad(a.mlp, 32 / a.G, 32)
+                        : act_stride_pad(a.mlp, a.threads / a.G, a.threads);
+  plan_rollout(a);   // the block rollouts take lanes and threads of their own
+  return SIMX_OK;
+}
+
+simx_status simx_launch_shape(simx_ctx* c, const simx_mlp* pol, int policy_mode,
+                              int32_t* host_out) {
+  if (!c || !host_out) return fail(SIMX_EINVAL, "ctx or host_out is NULL");
+  RolloutArgs a;
+  bool thread = false;
+  const simx_status v = rollout_plan(c, pol, policy_mode, a, thread);
+  if (v != SIMX_OK) return v;
   host_out[0] = thread ? 1 : 0;
   host_out[1] = thread ? 1 : a.G;
   host_out[2] = thread ? 128 : a.threads;
-  host_out[3] = (!thread && net) ? mlp_warp_of(route, a.G, pol) : 0;
-  host_out[4] = 0;
-  host_out[5] = 0;
-  if (!thread && net) {  // the launch's forward plans (no repack needed)
-    a.mlp_warp = host_out[3];
-    a.mlp.n_layers = pol->n_layers;
-    for (int l = 0; l <= pol->n_layers; ++l) {
-      a.mlp.dims[l] = pol->dims[l];
-      a.mlp.npad[l] = l ? round_up(pol->dims[l], 4) : pol->dims[0];
-    }
-    a.mlp.grid = pol->grid;
-    act_layout(mlp_maxdim(pol), (int)a.n_actions, a.maxd4, a.apad);
-    a.bs_pad = a.mlp_warp ? act_stride_pad(a.mlp, 32 / a.G, 32)
-                          : act_stride_pad(a.mlp, a.threads / a.G, a.threads);
-    plan_rollout(a);
-    host_out[1] = a.G;       // the block rollouts take their own
-    host_out[2] = a.threads;
-    if (a.fwd.on) host_out[3] = 0;
-    host_out[4] = a.tc.on;
-    host_out[5] = a.stage.on || a.fwd.on;
-  }
+  host_out[3] = a.mlp_warp && !a.fwd.on;
+  host_out[4] = a.tc.on;
+  host_out[5] = a.stage.on || a.fwd.on;
+  return SIMX_OK;
+}
+
+simx_status simx_rollout_kernel(simx_ctx* c, const simx_mlp* pol, int policy_mode, int32_t* host_out) {
+  if (!c || !host_out) return fail(SIMX_EINVAL, "ctx or host_out is NULL");
+  RolloutArgs a;
+  bool thread = false;
+  const simx_status v = rollout_plan(c, pol, policy_mode, a, thread);
+  if (v != SIMX_OK) return v;
+  host_out[0] = thread ? 1 : !a.fwd.on ? 0 : c->cfg.mode == SIMX_MODE_ROUTE ? 2 : 3;
+  host_out[1] = a.tc.on ? 4 : a.fwd.on ? (a.fwd.resident ? 3 : 2) : a.stage.on ? 1 : 0;
   return SIMX_OK;
 }
 
@@ -645,6 +660,20 @@ static simx_status policy_forward_check(const simx_mlp* pol, const float* d_obs,
   if (v != SIMX_OK) return v;
   if (d_value && !pol->has_value) return fail(SIMX_EINVAL, "d_value given but the policy has no value row");
   return SIMX_OK;
+}
+
+int32_t simx_forward_columns(const simx_mlp* pol, int64_t n) {
+  if (n < 1 || validate_mlp(pol, 0, 0) != SIMX_OK) return -1;
+  PolicyArgs p;
+  std::memset(&p, 0, sizeof(p));
+  p.mlp.n_layers = pol->n_layers;
+  for (int l = 0; l <= pol->n_layers; ++l) {
+    p.mlp.dims[l] = pol->dims[l];
+    p.mlp.npad[l] = l ? round_up(pol->dims[l], 4) : pol->dims[0];
+  }
+  p.mlp.n_actions = pol->dims[pol->n_layers] - (pol->has_value ? 1 : 0);
+  p.n = n;
+  return plan_policy_block(p) ? 1 << p.fwd.ne_shift : 0;
 }
 
 simx_status policy_forward(const simx_mlp* pol, const float* d_obs, int64_t ld, int64_t n,
@@ -761,16 +790,28 @@ static simx_status loss_args(const simx_mlp* pol, const simx_rollout* buf, int64
   return SIMX_OK;
 }
 
-size_t ppo_loss_grad_workspace_size(const simx_mlp* pol, int64_t n) {
-  if (!pol || pol->n_layers < 1 || pol->n_layers > SIMX_MAX_LAYERS || n < 1) return 0;
-  LossArgs a;
+// The part of the arguments that a loss call's kernel and workspace depend on.
+static bool loss_shape(const simx_mlp* pol, int64_t n, LossArgs& a) {
+  if (!pol || pol->n_layers < 1 || pol->n_layers > SIMX_MAX_LAYERS || n < 1) return false;
   std::memset(&a, 0, sizeof(a));
   a.n_layers = pol->n_layers;
   for (int l = 0; l <= pol->n_layers; ++l) a.dims[l] = pol->dims[l];
   for (int l = 0; l < pol->n_layers; ++l) a.act[l] = (l + 1 < pol->n_layers) ? pol->act[l] : -1;
   a.grid = pol->grid ? 1 : 0;
   a.n = n;
-  return loss_workspace_bytes(a);
+  return true;
+}
+
+size_t ppo_loss_grad_workspace_size(const simx_mlp* pol, int64_t n) {
+  LossArgs a;
+  return loss_shape(pol, n, a) ? loss_workspace_bytes(a) : 0;
+}
+
+int32_t simx_loss_kernel(const simx_mlp* pol, int64_t n, int precision) {
+  LossArgs a;
+  if (!loss_shape(pol, n, a)) return -1;
+  a.precision = precision;
+  return loss_path(a);
 }
 
 simx_status ppo_loss_grad(const simx_mlp* pol, const simx_rollout* buf, int64_t n_rows_per_step,

@@ -184,6 +184,10 @@ struct LossArgs {
   int gx[SIMX_MAX_LAYERS];   // grid policy: input grid exponent of layer l
 };
 size_t loss_workspace_bytes(const LossArgs& a);
+// The kernels that a call takes (loss.cu): the GEMM pipeline, or those of loss_fused.cu,
+// loss_block.cu, loss_tc.cu, loss_wide.cu; -1: refused.
+enum LossPath : int { LOSS_GEMM = 0, LOSS_FUSED = 1, LOSS_BLOCK = 2, LOSS_TC = 3, LOSS_WIDE = 4 };
+int loss_path(const LossArgs& a);
 // W_l as [K][npad] transposed and [N][kpad] copies, zero padded, every layer in one launch
 struct LossPack {
   const float* W[SIMX_MAX_LAYERS];

@@ -98,6 +98,9 @@ SIGNATURES = [
     ("sim_step_batched", C.c_int, [P, P, P, C.c_int, P, I64, P, P, P, P, P]),
     ("rollout_collect", C.c_int, [P, P, C.c_int, I32, P, P]),
     ("simx_launch_shape", C.c_int, [P, P, C.c_int, P]),
+    ("simx_rollout_kernel", C.c_int, [P, P, C.c_int, P]),
+    ("simx_forward_columns", C.c_int32, [P, I64]),
+    ("simx_loss_kernel", C.c_int32, [P, I64, C.c_int]),
     ("policy_forward", C.c_int, [P, P, I64, I64, C.c_int, U64, U32, U32, P, P, P, P, P]),
     ("policy_forward_workspace_size", SZ, [P]),
     ("policy_forward_ws", C.c_int, [P, P, I64, I64, C.c_int, U64, U32, U32, P, P, P, P, P, SZ, P]),
@@ -308,6 +311,15 @@ class Sim:
         return dict(kernel="thread" if out[0] else "fused", lanes=out[1], threads=out[2],
                     mlp_warp=bool(out[3]), tensor_cores=bool(out[4]), staged=bool(out[5]))
 
+    def rollout_kernel(self, policy_mode: str, policy: Policy = None) -> tuple:
+        """Which kernel that launch is (simx_rollout_kernel): ("lanes", "thread", "route" or
+        "single", where its forward reads the weights)."""
+        out = (C.c_int32 * 2)()
+        _check(lib().simx_rollout_kernel(self._h, C.byref(policy.c) if policy else None,
+                                         POLICY[policy_mode], out))
+        return (("lanes", "thread", "route", "single")[out[0]],
+                ("l1", "staged", "streamed", "resident", "tensor_cores")[out[1]])
+
     def stats(self) -> dict:
         c = Counters()
         _check(lib().sim_stats(self._h, C.byref(c)))
@@ -389,6 +401,17 @@ def returns_baseline(x, adv_out, mean_out, workspace, stream=None):
 
 def ppo_loss_grad_workspace_size(policy: Policy, n: int) -> int:
     return lib().ppo_loss_grad_workspace_size(C.byref(policy.c), n)
+
+
+def forward_columns(policy: Policy, n: int) -> int:
+    """Columns per block of policy_forward's block forward, 0 for its lane-group kernel."""
+    return lib().simx_forward_columns(C.byref(policy.c), n)
+
+
+def loss_kernel(policy: Policy, n: int, precision: str = "fp32") -> str:
+    """Which kernel ppo_loss_grad takes for n rows (simx_loss_kernel)."""
+    k = lib().simx_loss_kernel(C.byref(policy.c), n, PRECISION[precision])
+    return ("gemm", "fused", "block", "tc", "wide")[k] if k >= 0 else "refused"
 
 
 def ppo_loss_grad(policy: Policy, buf: dict, ret, adv, idx, n: int, algo: str, clip_eps: float,

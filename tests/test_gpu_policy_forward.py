@@ -36,6 +36,9 @@ def test_policy_forward(n, dims, acts, mode):
     obs = (rng.standard_normal((dims[0], n)) * np.exp(rng.uniform(-8, 4, (dims[0], n)))).astype(np.float32)
     pol = simx.Policy([torch.from_numpy(w).cuda() for w in Ws], [torch.from_numpy(b).cuda() for b in bs],
                       True, acts)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    block = 64 if n > 48 * sms else 32 if n > 32 * sms else 16 if n > 14 * sms else 8
+    assert simx.forward_columns(pol, n) == (0 if dims[-1] == 251 else block)
     A = dims[-1] - 1
     ld = n + 5
 

@@ -35,12 +35,13 @@ def _policy(simx, name, seed=7):
     return pol, (Ws, bs, hv, acts)
 
 
-def _run(name, cfg, H, mode, seed=None, trace=True):
+def _run(name, cfg, H, mode, seed=None, trace=True, kernel=None):
     simx = _simx()
     seed = W.SEED[name] if seed is None else seed
     E = cfg["n_envs"]
     pol, host = _policy(simx, name) if mode in ("sample", "argmax") else (None, None)
     sim = simx.Sim(cfg)
+    assert kernel in (None, sim.rollout_kernel(mode, pol)[0])
     sim.reset(seed)
     buf = simx.alloc_rollout(E, sim.D, H, has_value=bool(host and host[2]), trace=trace)
     sim.rollout(mode, H, buf, pol)
@@ -88,14 +89,17 @@ def test_rollout_matches_oracle(name, mk, H, mode):
     _assert_same(got, ref, W.MLP_SHAPES[name][1])
 
 
+@pytest.mark.parametrize("stage", ["", "0"], ids=["default", "lane-groups"])
 @pytest.mark.parametrize("lanes", [8, 16, 32])
 @pytest.mark.parametrize("name,mk,H,mode", [c for c in CASES if c[0] != "c1"] +
                          [("c1", lambda: W.c1(23), 1500, "sample")],
                          ids=[c[0] for c in CASES if c[0] != "c1"] + ["c1"])
-def test_rollout_every_lane_width(name, mk, H, mode, lanes, monkeypatch):
-    """The same results whichever number of lanes (8, 16, 32) serves an env."""
+def test_rollout_every_lane_width(name, mk, H, mode, lanes, stage, monkeypatch):
+    """The same results whichever number of lanes (8, 16, 32) serves an env: threads per env of the
+    block rollouts where these take the forced shape, and lane groups (SIMX_STAGE=0)."""
     monkeypatch.setenv("SIMX_LANES", str(lanes))
-    got, ref, st, code = _run(name, mk(), min(H, 300), mode)
+    monkeypatch.setenv("SIMX_STAGE", stage)
+    got, ref, st, code = _run(name, mk(), min(H, 300), mode, kernel="lanes" if stage else None)
     assert st == 0 and code == 0
     _assert_same(got, ref, W.MLP_SHAPES[name][1])
 

@@ -69,6 +69,8 @@ def test_route_rollout(cfg, hidden, acts, mode, H, request, monkeypatch):
         sim.reset(0xA11)
         shape = sim.launch_shape(mode, pol)
         assert shape["staged"] == (stage == "1") and shape["kernel"] == "fused"
+        kernel, weights = sim.rollout_kernel(mode, pol)
+        assert (kernel, weights) == ("route", "streamed") if stage == "1" else kernel == "lanes"
         buf = simx.alloc_rollout(E, sim.D, H, has_value=True, trace=True)
         sim.rollout(mode, H, buf, pol)
         nxt = torch.empty((sim.D, E), device="cuda")

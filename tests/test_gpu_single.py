@@ -64,6 +64,10 @@ def test_single_rollout(cfg, hidden, acts, mode, H, new, request, monkeypatch):
         sim = simx.Sim(cfg)
         sim.reset(0xB22)
         assert sim.launch_shape(mode, pol)["staged"] == (new and stage == "")
+        kernel, weights = sim.rollout_kernel(mode, pol)
+        assert kernel == ("single" if new and stage == "" else "lanes")
+        if kernel == "single":
+            assert weights == ("streamed" if "streamed" in request.node.callspec.id else "resident")
         buf = simx.alloc_rollout(E, sim.D, H, has_value=True, trace=True)
         sim.rollout(mode, H, buf, pol)
         nxt = torch.empty((sim.D, E), device="cuda")

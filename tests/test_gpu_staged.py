@@ -1,24 +1,22 @@
-"""The block-wide FP32 policy forward with its weights streamed through shared memory
-(Sec. 4.2 policy inside the fused step): one thread keeps two stages of weight rows in
-flight with bulk copies, every thread runs a register tile of up to 4 envs x 8 outputs.
+"""The block-wide FP32 policy forward with its weights streamed through shared memory (Sec. 4.2
+policy inside the fused step) at full sizes and forced shapes: two stages of weight rows in flight
+with bulk copies, register tiles of envs x outputs.  FP32 policies run it in the router's block
+rollout (or the single server's, there with the weights resident where they fit); a grid policy with
+the staging forced and the tensor-core forward off runs the lane-group kernel's staged form.
 
-Every output is still the fma chain from 0 over k in order, then + bias, the activation
-and (grid policies) the grid rounding, so the staged launch must give the unstaged
-launch's bits (SIMX_STAGE=0) on every env, and the oracle's on sampled envs (actions,
-traces, done flags, observations, rewards, log-probabilities, values, final state).
-Each case asserts the launch shape it means to cover:
+Every output is the fma chain from 0 over k in order, then + bias, the activation and (grid
+policies) the grid rounding, so the launch must give the bits of the weights read through L1
+(SIMX_STAGE=0) on every env, and the oracle's on sampled envs (actions, traces, done flags,
+observations, rewards, log-probabilities, values, final state).  Each case asserts the launch shape
+and the kernel it means to cover:
 
-* c4 at 65,536 envs (4x8 tiles for the 256-wide layers, 2x4 for the 49 outputs; 256-thread
-  blocks), 64 steps;
-* c3 at 16,384 envs (2x8 tiles, 1x4 for the 17 outputs; 128-thread blocks);
-* the paper's network (c1p: identity and GELU layers, five layers down to 4 wide) with
-  staging forced on small weights, in 256-thread blocks;
-* a c3 grid policy with staging forced and the tensor-core forward off: the grid
-  rounding in the staged epilogue;
-* c4 at 1,003 envs in 128-thread blocks (8 lanes, 4 KB stages): a last block with 11
-  envs;
-* c4 at 65,536 envs with 16 lanes per env (2x8 tiles, 1x4 for the 49 outputs, 16 envs per
-  256-thread block);
+* c4 at 65,536 envs in 256-thread blocks, 64 steps;
+* c3 at 16,384 envs in 128-thread blocks;
+* the paper's network (c1p: identity and GELU layers, five layers down to 4 wide) in 256-thread
+  blocks;
+* a c3 grid policy: the grid rounding in the lane-group kernel's staged epilogue;
+* c4 at 1,003 envs in 128-thread blocks (8 threads per env): a last block with 11 envs;
+* c4 at 65,536 envs with 16 threads per env (16 envs per 256-thread block);
 * c3t, trace replay (gaps, types and costs from a trace), at 16,384 envs;
 * single steps (sim_step_batched: one launch per step, so the weight pipeline starts and
   drains every launch) against rollout_collect, c4 at 4,096 envs in 256-thread blocks.
@@ -71,6 +69,7 @@ def _rollout(simx, cfg, host, mode, H, seed, stage, monkeypatch):
                       [torch.from_numpy(b).cuda() for b in bs], hv, acts, grid=gx)
     sim = simx.Sim(cfg)
     shape = sim.launch_shape(mode, pol)
+    shape["path"] = sim.rollout_kernel(mode, pol)
     sim.reset(seed)
     buf = simx.alloc_rollout(cfg["n_envs"], sim.D, H, has_value=hv, trace=True)
     sim.rollout(mode, H, buf, pol)
@@ -82,22 +81,23 @@ def _rollout(simx, cfg, host, mode, H, seed, stage, monkeypatch):
     return shape, buf, state
 
 
-# name, envs, steps, mode, grid policy, SIMX_THREADS, SIMX_LANES, SIMX_STAGE, threads
+# name, envs, steps, mode, grid policy, SIMX_THREADS, SIMX_LANES, SIMX_STAGE, threads, kernel
+ROUTE = ("route", "streamed")
 CASES = [
-    ("c4", 65536, 64, "sample", False, None, None, "", 256),
-    ("c3", 16384, 96, "sample", False, None, None, "", 128),
-    ("c1p", 4096, 300, "sample", False, "256", None, "1", 256),
-    ("c3", 16384, 64, "argmax", True, None, None, "1", 128),
-    ("c4", 1003, 200, "sample", False, "128", "8", "", 128),
-    ("c4", 65536, 32, "sample", False, None, "16", "", 256),
-    ("c3t", 16384, 64, "sample", False, None, None, "", 128),
+    ("c4", 65536, 64, "sample", False, None, None, "", 256, ROUTE),
+    ("c3", 16384, 96, "sample", False, None, None, "", 128, ROUTE),
+    ("c1p", 4096, 300, "sample", False, "256", None, "1", 256, ("single", "resident")),
+    ("c3", 16384, 64, "argmax", True, None, None, "1", 128, ("lanes", "staged")),
+    ("c4", 1003, 200, "sample", False, "128", "8", "", 128, ROUTE),
+    ("c4", 65536, 32, "sample", False, None, "16", "", 256, ROUTE),
+    ("c3t", 16384, 64, "sample", False, None, None, "", 128, ROUTE),
 ]
 
 
-@pytest.mark.parametrize("name,E,H,mode,grid,threads,lanes,stage,expect", CASES,
+@pytest.mark.parametrize("name,E,H,mode,grid,threads,lanes,stage,expect,path", CASES,
                          ids=["c4", "c3", "c1p-forced", "c3-grid-forced", "c4-ragged", "c4-16-lanes",
                               "c3t"])
-def test_staged_forward(name, E, H, mode, grid, threads, lanes, stage, expect, monkeypatch):
+def test_staged_forward(name, E, H, mode, grid, threads, lanes, stage, expect, path, monkeypatch):
     simx = _simx()
     if threads:
         monkeypatch.setenv("SIMX_THREADS", threads)
@@ -109,9 +109,9 @@ def test_staged_forward(name, E, H, mode, grid, threads, lanes, stage, expect, m
     seed = 0x57A6 + E
     shape, buf, state = _rollout(simx, cfg, host, mode, H, seed, stage, monkeypatch)
     assert shape["kernel"] == "fused" and shape["threads"] == expect and not shape["mlp_warp"]
-    assert shape["staged"] and not shape["tensor_cores"]
+    assert shape["staged"] and not shape["tensor_cores"] and shape["path"] == path
     shape0, buf0, state0 = _rollout(simx, cfg, host, mode, H, seed, "0", monkeypatch)
-    assert not shape0["staged"]
+    assert not shape0["staged"] and shape0["path"] == ("lanes", "l1")
     # every env: the unstaged forward's bits
     for k in buf:
         assert torch.equal(buf[k], buf0[k]), k
@@ -144,6 +144,7 @@ def test_staged_single_steps_equal_the_rollout(monkeypatch):
     sim = simx.Sim(cfg)
     shape = sim.launch_shape("sample", pol)
     assert shape["staged"] and shape["threads"] == 256 and shape["lanes"] == 8
+    assert sim.rollout_kernel("sample", pol) == ROUTE
     sim.reset(seed)
     buf = simx.alloc_rollout(E, sim.D, H, has_value=hv)
     sim.rollout("sample", H, buf, pol)
