@@ -627,7 +627,7 @@ __device__ __forceinline__ int sample_action(const DevMlp& m, const float* z, in
       float S = 0.0f;
       for (int i = 0; i < A; ++i) S = __fadd_rn(S, scratch[i]);
       if (mode == SIMX_POLICY_ARGMAX) {
-        a = ai;
+        a = ai < A ? ai : 0;   // (no logit above -inf)
       } else {
         const U4 w = philox(step, env, kStreamPolicy, 0u, key0, key1);
         const float thr = __fmul_rn(u_open1(w.x), S);

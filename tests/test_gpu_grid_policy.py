@@ -137,3 +137,28 @@ def test_grid_policy_validation():
                        0.0, grad, stats, ws)
     torch.cuda.synchronize()
     assert torch.isfinite(grad).all() and torch.isfinite(stats).all()
+
+
+@pytest.mark.parametrize("lanes", ["", "8", "16", "32"])
+@pytest.mark.parametrize("logit", [float("nan"), float("-inf")])
+def test_no_logit_above_minus_infinity(lanes, logit, monkeypatch):
+    """ARGMAX over logits of which none is above -inf (a diverged policy's) takes action 0 on every
+    kernel; an index of nothing would be read with."""
+    simx = _simx()
+    monkeypatch.setenv("SIMX_LANES", lanes) if lanes else monkeypatch.delenv("SIMX_LANES", raising=False)
+    dims, hv = W.mlp_dims("c3")
+    gx, ew = [4, 7, 7], [6] * 3
+    Ws, bs = W.grid_weights(dims, 5, gx, ew)
+    bs[-1] = np.full_like(bs[-1], logit)
+    E = 300
+    for grid in (gx, None):
+        pol = simx.Policy([torch.from_numpy(w).cuda() for w in Ws], [torch.from_numpy(b).cuda() for b in bs],
+                          hv, grid=grid)
+        sim = simx.Sim(W.c3(E))
+        sim.reset(1)
+        buf = simx.alloc_rollout(E, sim.D, 5, has_value=hv)
+        sim.rollout("argmax", 5, buf, pol)
+        torch.cuda.synchronize()
+        assert sim.last_status() == (0, 0)
+        assert int(buf["action"].max()) == 0
+        sim.close()
