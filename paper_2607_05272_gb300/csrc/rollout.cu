@@ -875,9 +875,10 @@ k_rollout(const __grid_constant__ RolloutArgs A) {
   uint32_t* tc_tbase = reinterpret_cast<uint32_t*>(tsm + A.tc.bar_off + 8);
   if (tc) tcf::setup(A, tsm, tc_tbase);
   const uint32_t tc_tmem = tc ? *tc_tbase : 0u;
-  // fp32 policies with staged weights: the launch's pipeline of weight chunks (not
-  // instantiated for 32 lanes per env, whose blocks hold at most 8 envs)
-  const bool stg = G != 32 && !WARP && !tc && A.stage.on && use_mlp;
+  // grid policies with staged weights: the launch's pipeline of weight chunks (not
+  // instantiated for 32 lanes per env, whose blocks hold at most 8 envs, nor for fp32
+  // policies, whose block rollouts stream or keep theirs)
+  const bool stg = GRID && G != 32 && !WARP && !tc && A.stage.on && use_mlp;
   StagePipe sp;
   sp.stages = reinterpret_cast<float*>(tsm + A.stage.off);
   sp.full = reinterpret_cast<uint64_t*>(tsm + A.stage.bar_off);
@@ -908,7 +909,7 @@ k_rollout(const __grid_constant__ RolloutArgs A) {
         Z = tcf::forward(A, tsm, tc_tmem, X0, X1, B, Bs, tc_phase, tc_timeout);
         if (tc_timeout) s.status |= SIMX_DEV_TC_TIMEOUT;
       } else if (stg) {
-        Z = mlp_forward_staged<GRID>(A.mlp, A.stage, sp, X0, X1, B, Bs);
+        Z = mlp_forward_staged(A.mlp, A.stage, sp, X0, X1, B, Bs);
         if (*sp.flag) s.status |= SIMX_DEV_COPY_TIMEOUT;
       } else {
         Z = WARP ? mlp_forward_warp<GRID>(A.mlp, X0, X1, 32 / G, Bs, (int)(threadIdx.x / 32) * (32 / G))
@@ -1376,8 +1377,8 @@ static bool stage_tiles(const DevMlp& m, int B, int threads, StagePlan& P) {
   return true;
 }
 
-// The staged forward's plan (fp32 block-wide forwards of 8 or 16 lanes per env whose
-// weights are large): two
+// The staged forward's plan (block-wide forwards of grid policies, 8 or 16 lanes per env,
+// whose weights are large): two
 // stages of the largest chunk size in 16, 12, 8, 4 KB that keeps the blocks per SM of the
 // unstaged launch of `kfn`.  Sets a.stage (and a.bs_pad = 4, so the activation rows stay
 // 16-byte aligned) and returns the dynamic shared memory; otherwise leaves a.stage off.
@@ -1386,7 +1387,7 @@ static size_t plan_stage_forward(RolloutArgs& a, int B, const void* kfn) {
   const DevMlp& m = a.mlp;
   const size_t plain = env_smem(a, B);
   const bool net = a.policy_mode == SIMX_POLICY_SAMPLE || a.policy_mode == SIMX_POLICY_ARGMAX;
-  if (!net || a.mlp_warp || a.tc.on || a.G == 32) return plain;
+  if (!net || !m.grid || a.mlp_warp || a.tc.on || a.G == 32) return plain;
   int force = -1;
   if (const char* f = getenv("SIMX_STAGE"))
     if (f[0]) force = f[0] == '0' ? 0 : 1;

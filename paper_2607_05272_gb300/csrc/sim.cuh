@@ -49,8 +49,8 @@ struct DevMlp {
   int gx[SIMX_MAX_LAYERS];
 };
 
-// The FP32 block-wide forward with its weights staged in shared memory (fp32 policies
-// whose weights L1 does not hold): one thread streams each layer's rows, in chunks of
+// The lane groups' block-wide FP32 forward of a grid policy with its weights staged in shared
+// memory (policies whose weights L1 does not hold): one thread streams each layer's rows, in chunks of
 // rpc[l] rows, into S stages of cb bytes with bulk copies; every thread reads its
 // register tile's weights (te[l] envs x to[l] outputs) from the stage.  The chunk
 // sequence of one forward (layer 0's, then layer 1's, ...) repeats every step, so the
@@ -68,9 +68,9 @@ struct StagePlan {
   int te[SIMX_MAX_LAYERS], to[SIMX_MAX_LAYERS];   // register tile: envs x outputs
 };
 
-// Policies of at least this many fp32 weight bytes have their weights staged in shared
-// memory by default (SIMX_STAGE=0 / 1 turns staging off / on for any size); L1 holds smaller
-// ones.
+// Router policies of at least this many fp32 weight bytes take the block rollout, and grid
+// policies have their weights staged in shared memory, by default (SIMX_STAGE=0 / 1 turns that
+// off / on for any size); L1 holds smaller ones.
 constexpr size_t kStageMinBytes = 64 * 1024;
 
 // The block forward of fwd_block.cuh: S stages of cb bytes, chunks of rpc[l] weight rows,
@@ -79,13 +79,14 @@ constexpr size_t kStageMinBytes = 64 * 1024;
 struct FwdPlan {
   int on, big;                 // big: the kernel with 8 x 8 tiles
   int S, n;
-  uint32_t cb, off, bar_off;   // stages, then 2 S mbarriers (8 B each) and the timeout flag (4 B)
+  uint32_t cb, off, bar_off;   // stages, then 2 S mbarriers (8 B each), the timeout flag, the producer's place
   uint32_t st_off, red_off;    // env words, softmax partials
   int ld, ex_row;              // activation row stride, first row of the exponentials
   int ne_shift;                // log2 of the envs per block
   uint32_t bias_off;           // the biases of every layer, layer l's from float boff[l]
   int boff[SIMX_MAX_LAYERS];
-  uint32_t part_off;           // partial results of the servers, S_PARTS words per thread
+  uint32_t part_off;           // rollout_route.cu: the servers' partial results, Q_WORDS words per thread;
+                               // rollout_single.cu: the envs' counter
   int sms;                     // blocks of one wave index (rotates the warps' roles)
   int side_layer, side_vt;     // layer beside whose products side work runs (-1: none), from thread
   int rpc[SIMX_MAX_LAYERS], cnt[SIMX_MAX_LAYERS];
@@ -378,7 +379,8 @@ __device__ __forceinline__ float* mlp_forward_warp(const DevMlp& m, float* X0, f
 }
 
 // ---------------------------------------------------------------------------
-// The block-wide forward with the weights staged in shared memory (StagePlan).  Thread 0
+// The grid policy's block-wide forward with the weights staged in shared memory (StagePlan; fp32
+// policies take the block forward of fwd_block.cuh).  Thread 0
 // keeps S chunks of weight rows in flight (bulk copies completing on one mbarrier per
 // stage); every thread owns one register tile of TE envs x TO outputs of the layer and,
 // per chunk, waits for its stage, runs its rows k in order (paired fmas, f2_fma) and
@@ -435,7 +437,7 @@ __device__ __forceinline__ void stage_drain(const StagePlan& P, const StagePipe&
 }
 
 // One layer of the staged forward; returns the chunks consumed so far.
-template <int TE, int TO, bool GRID>
+template <int TE, int TO>
 __device__ __forceinline__ uint32_t layer_staged(const DevMlp& m, const StagePlan& P,
                                                      StagePipe p, int l, const float* X, float* Y,
                                                      int B, int ld, int gq) {
@@ -518,7 +520,7 @@ __device__ __forceinline__ uint32_t layer_staged(const DevMlp& m, const StagePla
     }
     if (act == 2)
       for (int o4 = 0; o4 < TO; o4 += 4) gelu_tile(Y + TE * eb, ld, TO * ob + o4, N, TE);
-    if (GRID && gq >= 0)
+    if (gq >= 0)
       for (int o4 = 0; o4 < TO; o4 += 4) grid_tile(Y + TE * eb, ld, TO * ob + o4, N, TE, gq);
   }
   return p.cc;
@@ -527,26 +529,23 @@ __device__ __forceinline__ uint32_t layer_staged(const DevMlp& m, const StagePla
 // Forward through every layer with staged weights (the same buffers and result as
 // mlp_forward_block).  Contains the block barriers.  Inlined: as an out-of-line call it
 // ran the c4 policy 26 % slower inside the rollout.
-template <bool GRID>
 __device__ __forceinline__ float* mlp_forward_staged(const DevMlp& m, const StagePlan& P,
                                                     StagePipe& p, float* X0, float* X1, int B,
                                                     int ld) {
   float* in = X0;
   float* out = X1;
   __syncthreads();
-  if (GRID) {
-    grid_rows(X0, m.dims[0], B, ld, m.gx[0], threadIdx.x, blockDim.x);
-    __syncthreads();
-  }
+  grid_rows(X0, m.dims[0], B, ld, m.gx[0], threadIdx.x, blockDim.x);
+  __syncthreads();
   for (int l = 0; l < m.n_layers; ++l) {
-    const int gq = (GRID && l + 1 < m.n_layers) ? m.gx[l + 1] : -1;
+    const int gq = l + 1 < m.n_layers ? m.gx[l + 1] : -1;
     switch (P.te[l] * 16 + P.to[l]) {
-      case 4 * 16 + 8: p.cc = layer_staged<4, 8, GRID>(m, P, p, l, in, out, B, ld, gq); break;
-      case 2 * 16 + 8: p.cc = layer_staged<2, 8, GRID>(m, P, p, l, in, out, B, ld, gq); break;
-      case 4 * 16 + 4: p.cc = layer_staged<4, 4, GRID>(m, P, p, l, in, out, B, ld, gq); break;
-      case 2 * 16 + 4: p.cc = layer_staged<2, 4, GRID>(m, P, p, l, in, out, B, ld, gq); break;
-      case 1 * 16 + 8: p.cc = layer_staged<1, 8, GRID>(m, P, p, l, in, out, B, ld, gq); break;
-      default: p.cc = layer_staged<1, 4, GRID>(m, P, p, l, in, out, B, ld, gq); break;
+      case 4 * 16 + 8: p.cc = layer_staged<4, 8>(m, P, p, l, in, out, B, ld, gq); break;
+      case 2 * 16 + 8: p.cc = layer_staged<2, 8>(m, P, p, l, in, out, B, ld, gq); break;
+      case 4 * 16 + 4: p.cc = layer_staged<4, 4>(m, P, p, l, in, out, B, ld, gq); break;
+      case 2 * 16 + 4: p.cc = layer_staged<2, 4>(m, P, p, l, in, out, B, ld, gq); break;
+      case 1 * 16 + 8: p.cc = layer_staged<1, 8>(m, P, p, l, in, out, B, ld, gq); break;
+      default: p.cc = layer_staged<1, 4>(m, P, p, l, in, out, B, ld, gq); break;
     }
     __syncthreads();
     float* t = in;
