@@ -203,6 +203,7 @@ size_t loss_block_workspace(const LossArgs& a);
 cudaError_t launch_loss_block(const LossArgs& a, void* ws, size_t ws_bytes, cudaStream_t s);
 // loss_fused.cu
 bool loss_fused_fits(const LossArgs& a);
+int loss_fused_tile(const LossArgs& a);       // rows of its tiles
 int64_t loss_fused_rows(const LossArgs& a);   // rows that the busiest block takes
 size_t loss_fused_workspace(const LossArgs& a);
 cudaError_t launch_loss_fused(const LossArgs& a, void* ws, size_t ws_bytes, cudaStream_t s);

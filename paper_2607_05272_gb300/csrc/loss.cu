@@ -369,12 +369,16 @@ static WsLayout layout(const LossArgs& a) {
   return w;
 }
 
-// The block kernel where its one tile per SM has fewer rows than the fused kernel's busiest block
-// walks (5000 rows of 13-128-128-17: 40 against 64; at 4096 both have 32 and the fused one is the
-// faster, 42 us against 49), and only within the scratch that the call has always asked for.
+// The block kernel for policies whose fused kernel walks 32-row tiles, alone on its SM, where one
+// tile per SM has fewer rows than the busiest of its blocks walks (5000 rows of 13-128-128-17: 40
+// against 64, 60 us against 73; at 4096 both have 32 and the fused one is the faster, 43 us against
+// 49), and only within the scratch that the call has always asked for: a partial per tile, so no
+// more tiles than the fused kernel has blocks.  That leaves 1 to 8 rows (one tile either way, 35 us
+// against 40) and 33 to 56 rows per SM.  With 64-row tiles and resident weights the fused kernel is
+// the faster at any size (16-64-64-12, 8 rows: 31 us against 35).
 static bool loss_block_taken(const LossArgs& a) {
   const int R = loss_block_rows(a);
-  return R > 0 && loss_fused_fits(a) && R < loss_fused_rows(a) &&
+  return R > 0 && loss_fused_fits(a) && loss_fused_tile(a) == 32 && R < loss_fused_rows(a) &&
          loss_block_workspace(a) <= loss_fused_workspace(a);
 }
 

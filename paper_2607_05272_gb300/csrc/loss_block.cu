@@ -13,12 +13,14 @@
 // The block partials are summed in block order.
 //
 // What bounds it: latency between barriers (16 warps per SM issue in 36 % of the cycles; the top
-// stalls are shared-memory loads and barriers).  The fused kernel (loss_fused.cu) stages one
-// layer's weights at a time and holds dZ apart, which leaves 8 warps per SM on 32-row tiles: 8192
-// rows of 13-128-128-17 are two rounds of its blocks, 72 us, against one round here, 66 us (4865
-// rows: 70 against 60).  A second tile per block would add to a partial in L2 and measured slower
-// than the fused kernel (65,536 rows: 645 us against 406), as did equal rows per block (4096 rows:
-// 49 against 42), so those stay there.
+// stalls are the barriers, 3.0 cycles an instruction, and shared-memory loads, 2.5).  The fused kernel
+// (loss_fused.cu) stages one layer's weights at a time and holds dZ apart, which leaves 8 warps per
+// SM on 32-row tiles: above 32 rows per SM they are two rounds of its blocks, against one round here
+// (13-128-128-17 on 152 SMs: 4865 rows 73 us against 60, 8192 75 against 66).  A second tile per
+// block would add to a partial in L2 and measured slower than the fused kernel (65,536 rows: 645 us
+// against 420), as did equal rows per block (4096 rows: 49 against 43), so those stay there.  The
+// price of the range is that it is narrow: three layers of 98 to 128 at 33 to 56 rows per SM (see
+// loss_block_taken in loss.cu).
 #include <cstdint>
 
 #include "fwd_block.cuh"

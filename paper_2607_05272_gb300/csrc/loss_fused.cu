@@ -329,8 +329,9 @@ __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;\
 // whose weights do not stay in L1 beside one block's shared memory).  WS 2: every weight,
 // in both orders, stays in shared memory, in the place of the dZ buffers: dZ of a hidden
 // layer is written over its activations.  Through what two blocks leave of L1, the
-// 43 KB of 16-64-64-12 missed on every pass (its largest stall): 4096 rows 39.3 -> 31.9 us,
-// 262,144 rows 489 -> 408.  The products read the same values in the same order each way.
+// 43 KB of 16-64-64-12 missed on every pass (its largest stall): with dW still in pairs,
+// 4096 rows 39.3 -> 31.9 us, 262,144 rows 489 -> 408 (with dW in row order 32.3 and 411).  The
+// products read the same values in the same order each way.
 template <int R, int WS>
 __global__ void __launch_bounds__(kLThreads) k_loss_fused(const __grid_constant__ FusedLossArgs F) {
   constexpr int kLR = R, kLld = R + 4, kLanes = kLThreads / R;  // lanes per row in the head
@@ -676,6 +677,7 @@ void launch_pack_loss_w(const LossPack& p, cudaStream_t s) {
 }
 
 bool loss_fused_fits(const LossArgs& a) { return plan(a).ok; }
+int loss_fused_tile(const LossArgs& a) { return plan(a).R; }
 int64_t loss_fused_rows(const LossArgs& a) {
   const FusedPlan p = plan(a);
   const int64_t ntiles = (a.n + p.R - 1) / p.R;

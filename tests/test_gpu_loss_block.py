@@ -42,15 +42,19 @@ def test_block_loss_gradient_matches_oracle(name, algo, per_sm, over, kernel):
     _check(_simx(), name, algo, -(-n // 256), 256, n, None, kernel)
 
 
+@pytest.mark.parametrize("n,kernel", [(1, "block"), (8, "block"), (9, "fused")])
+def test_block_loss_gradient_of_few_rows(n, kernel):
+    _check(_simx(), "c3", "ppo", 4, 64, n, None, kernel)
+
+
 def test_block_loss_gradient_of_odd_widths():
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     _check(_simx(), "c3", "reinforce", -(-47 * sms // 101), 101, None, 100, "block")   # every row
 
 
 @pytest.mark.parametrize("name,algo,E,H,nmb,hidden,kernel", [
-    ("c2", "reinforce", 1, 1, None, None, "block"),   # up to 8 rows of any policy that fits
-    ("c2", "ppo", 4, 2, 8, None, "block"),
-    ("c2", "ppo", 4, 64, 9, None, "fused"),
+    ("c2", "reinforce", 1, 1, None, None, "fused"),   # one row
+    ("c2", "ppo", 4, 2, 8, None, "fused"),
     ("c2", "ppo", 16, 64, 64, None, "fused"),         # one full tile
     ("c2", "ppo", 16, 64, 65, None, "fused"),
     ("c2", "reinforce", 40, 512, 19457, None, "fused"),  # one block walks two tiles
@@ -59,6 +63,5 @@ def test_block_loss_gradient_of_odd_widths():
     ("c1", "ppo", 64, 400, 20000, None, "fused"),
 ])
 def test_resident_weights_loss_gradient_matches_oracle(name, algo, E, H, nmb, hidden, kernel):
-    """The fused kernel with every weight in shared memory, dZ over the activations, and the few rows
-    that take the block kernel before it."""
+    """The fused kernel with every weight in shared memory, dZ over the activations."""
     _check(_simx(), name, algo, E, H, nmb, hidden, kernel)
