@@ -13,10 +13,12 @@
 //   - the warps take the envs in turn to their next decision, 32 candidates at a time, a lane
 //     each, from a window of drawn candidates per env in shared memory, refilled 96 at a time.
 // The requests' rings are in shared memory too where they fit and the horizon pays for the copy.
-// What bounds it: each warp's dependent chain through its envs' candidates (about a third of the
-// step, another fifth waiting for the block's slowest), then the forward's short layers.  Measured
-// against the lane-group kernel, us per step: c2 at 4096 envs 20.8 -> 17.1, at 30,000 193 -> 80;
-// c2 with 65 actions at 65,000 418 -> 212; the paper's network at 4096 17.4 -> 14.6.
+// What bounds it: the dependent chains between the barriers, above all a warp's through its envs'
+// candidates, and the wait for the block's slowest (c2 at 4096 envs: 13.4 warps per SM issue in 38 %
+// of the cycles; the barrier is the largest stall, 3.0 cycles an instruction, then fixed latencies,
+// 1.8, and shared-memory loads, 1.1).  Measured against the lane-group kernel, us per step: c2 at
+// 4096 envs 20.0 -> 17.0 (from a fresh reset 19.7 -> 16.4), at 30,000 196 -> 80; c2 with 65 actions
+// at 65,000 421 -> 212; the paper's network at 4096 16.6 -> 14.4.
 #include <cstdint>
 #include <cstdlib>
 #include <cstring>
@@ -597,9 +599,9 @@ size_t plan_single(RolloutArgs& a) {
   for (int l = 0; l < m.n_layers; ++l) wbytes += (size_t)m.dims[l] * m.npad[l + 1] * sizeof(float);
   if (!forced) {
     // Up to one env per warp slot the lane-group kernel's 32 lanes per env are faster (c2 at 512
-    // envs 10.1 against 11.4 us per step, c1 at 1000 4.7 against 6.3), and so they are, with fewer
-    // lanes, for a policy too small to share (c1's 450 weights at 8000 envs: 10.1 against 15.5;
-    // at 65,000 57.5 against 55.5).  16 envs per block while two blocks per SM hold them all
+    // envs 9.4 against 11.4 us per step, c1 at 1000 4.7 against 6.3), and so they are, with fewer
+    // lanes, for a policy too small to share (c1's 450 weights at 8000 envs: 9.7 against 15.5;
+    // at 65,000 62.0 against 56.5).  16 envs per block while two blocks per SM hold them all
     // (c2 at 4096: 17.1 against 21.4 with 32), then 32 (at 30,000: 80 against 114).
     if (E <= 16 * sms || (wbytes < 4096 && E <= 256 * sms)) return 0;
     threads = 256;
