@@ -8,11 +8,12 @@ order, so these compare within tolerances derived from the arithmetic:
 * loss gradients, per tensor: ||g - g_ref|| <= 1e-5 ||g_ref||, per element:
   |g - g_ref| <= 1e-5 (|g_ref| + rms(g_ref)); the tensor-core (TF32-input) path is held
   to 1e-2 under the same definitions.
-Sizes span several blocks with ragged tails, plus the full c1 returns shape; every env
-count here (up to 40,000) takes the chunked two-pass returns kernel.  Env counts from
+Sizes span several blocks with ragged tails, plus the full c1 returns shape; returns here (env
+counts up to 40,000) take the chunked two-pass kernel, GAE from 16,384 envs the one whose chunks
+stay in registers (test_gpu_returns_once.py has its edges).  Env counts from
 65,536 that are a multiple of 4 take the one-pass four-envs-per-thread kernel instead;
 test_gpu_launch_shapes.py covers it at 65,536 and 262,144 envs (and 262,145, which
-falls back to the chunked one).
+falls back to the chunked ones).
 """
 import numpy as np
 import pytest
