@@ -1,7 +1,7 @@
 """Parity at the benchmark's full sizes, in the launch configurations bench.py times.
 
-* c2 as the benchmark runs it (4096 envs x 512 steps, 16 lanes per env, 64-thread blocks,
-  the benchmark's seed and weights): sampled envs, which the oracle reproduces one by one,
+* c2 as the benchmark runs it (4096 envs x 512 steps, the single server's block rollout with
+  16 envs per block, the benchmark's seed and weights): sampled envs, which the oracle reproduces one by one,
   bit for bit (records and final state).
 * The benchmark step's returns and mean baseline over all 2,097,152 rows against the fp64
   recurrence (within 1e-5 of the recurrence on absolute values), and its REINFORCE loss
@@ -41,6 +41,7 @@ def _c2_rollout(simx):
     pol = simx.Policy([torch.from_numpy(w).cuda() for w in Ws],
                       [torch.from_numpy(b).cuda() for b in bs], hv)
     sim = simx.Sim(cfg)
+    assert sim.rollout_kernel("sample", pol) == ("single", "resident")
     sim.reset(SEED_BENCH)
     buf = simx.alloc_rollout(E, sim.D, H, trace=True)
     sim.rollout("sample", H, buf, pol)

@@ -2,8 +2,8 @@
 (the exact dot product, an fp64 sum rounded once to fp32), through the C ABI.
 
 * Rollouts bit for bit (actions, log-probabilities, values, observations, rewards, final
-  state): c2 on the warp-local forward (16-64-64-12), c1p's GELU network on the block-wide
-  forward, and the c3 router; ragged env counts.
+  state): c2 on the lane groups' warp-local forward (16-64-64-12), c1p's GELU network on their
+  block-wide forward, and c3 on the router's block rollout; ragged env counts.
 * policy_forward at the premise's worst case: a hidden layer saturated at +-255 units
   feeding a fan-in-256 output layer with every mantissa at +-255 and the largest bias, so
   the kernel's fp32 FMA chains run up to 2^24 product units.
@@ -34,8 +34,9 @@ def _dev(simx, Ws, bs, hv, gx, acts=None):
                        [torch.from_numpy(b).cuda() for b in bs], hv, acts, grid=gx)
 
 
-@pytest.mark.parametrize("name,E", [("c2", 1000), ("c1p", 301), ("c3", 517)])
-def test_grid_rollout_matches_oracle(name, E):
+@pytest.mark.parametrize("name,E,kernel", [("c2", 1000, "lanes"), ("c1p", 301, "lanes"), ("c3", 517, "route")],
+                         ids=["c2-1000", "c1p-301", "c3-517"])
+def test_grid_rollout_matches_oracle(name, E, kernel):
     simx = _simx()
     cfg = W.CONFIGS[name](E)
     dims, hv = W.mlp_dims(name)
@@ -47,6 +48,8 @@ def test_grid_rollout_matches_oracle(name, E):
     pol = _dev(simx, Ws, bs, hv, gx, acts)
     H, seed = 48, 0x6A1D
     sim = simx.Sim(cfg)
+    assert sim.rollout_kernel("sample", pol)[0] == kernel
+    assert sim.launch_shape("sample", pol)["mlp_warp"] == (name == "c2")
     sim.reset(seed)
     buf = simx.alloc_rollout(E, sim.D, H, has_value=hv, trace=True)
     sim.rollout("sample", H, buf, pol)
