@@ -18,7 +18,7 @@
 // What bounds it: the dependent chains of a block's step (products, then softmax, draw, starts),
 // which the other blocks on the SM overlap.  c3 at 16,384 envs: 23.3 warps per SM issue in 55 % of
 // the cycles, the barrier the largest stall (2.8 cycles an instruction), the FMA pipes 26 % busy; its
-// kernel, 128 threads at 72 registers so that 7 blocks fit, spills 44 bytes.  Measured
+// kernel has 128 threads at 72 registers, without spills, so that 7 blocks fit.  Measured
 // against the lane-group kernel, us per step: c4 at 65,536 envs 427 -> 317, at 4096 59 -> 32, at 1000
 // 52 -> 20; c3 at 16,384 envs 49.5 -> 37.2, at 1000 12.2 -> 10.1; c3's env at 262,144 662 -> 444.
 #include <cstdint>
