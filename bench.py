@@ -412,9 +412,9 @@ class Clocks:
 # DRAM bytes (read + write) of one k_route launch of the benchmark workload, from an
 # ncu capture of the current kernel; None until one is taken, and to be re-measured (or
 # set back to None) whenever the rollout kernel changes.
-ROLLOUT_DRAM_BYTES = 407104512.0 + 4509971968.0
+ROLLOUT_DRAM_BYTES = 410956544.0 + 4510787840.0
 ROLLOUT_DRAM_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_route launch "
-                       "of this workload (407.1 MB + 4510.0 MB; profiles/k_route_c4_bench.md)")
+                       "of this workload (411.0 MB + 4510.8 MB; profiles/k_route_c4_bench.md)")
 
 
 def _peaks():
